@@ -1,0 +1,29 @@
+"""The stage kernel's strip reconstruction at the edges of its ranges: block
+extents below, at and above a strip's six cells and the default tiles, with
+every remainder of (extent + 2) / 6, against the oracle.  The bars are those
+of test_gpu_parity (rounding order only): 1e-12 in FP64, 1e-5 mixed."""
+import pytest
+
+import problems as pb
+from tests.test_gpu_parity import TOL64, TOLMIX, assert_parity, gb, one_step  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+BLOCKS = [(3, 4, 3), (5, 7, 4), (6, 10, 5), (8, 3, 7), (11, 5, 3), (16, 6, 4), (22, 9, 3)]
+
+
+@pytest.mark.parametrize("form,tol", [("fp64", TOL64), ("mixed", TOLMIX)])
+@pytest.mark.parametrize("recon", ["ppm", "minmod"])
+@pytest.mark.parametrize("nx", BLOCKS)
+def test_odd_blocks_3d(gb, nx, recon, form, tol):  # noqa: F811
+    g = pb.periodic_box(ndim=3).with_(nx=nx, nroot=(2, 2, 2), blocks=None, recon=recon)
+    s, o, _ = one_step(gb, g, pb.random_periodic_prims(g), form)
+    assert_parity(s.cons(), o.cons(), tol, f"{nx} {recon} {form}", g)
+
+
+@pytest.mark.parametrize("form,tol", [("fp64", TOL64), ("mixed", TOLMIX)])
+@pytest.mark.parametrize("nx", [(3, 5), (7, 3), (20, 13), (40, 9)])
+def test_odd_blocks_2d_torus(gb, nx, form, tol):  # noqa: F811
+    g = pb.torus_2d().with_(nx=(*nx, 1), nroot=(4, 4, 1), blocks=None)
+    s, o, _ = one_step(gb, g, pb.fm_torus_prims(g), form)
+    assert_parity(s.cons(), o.cons(), tol, f"{nx} {form}", g)
