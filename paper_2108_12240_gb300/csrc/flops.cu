@@ -71,7 +71,27 @@ template <int P> double to_double(Num<P> x) { return (double)x.v; }
 using N64 = Num<64>;
 using N32 = Num<32>;
 
+// halving is an exponent step in the kernels: no operation is counted
+inline N64 half_t(N64 x) {
+  N64 r;
+  r.v = 0.5 * x.v;
+  return r;
+}
+inline void limit_dev(N64& l, N64& r) {  // integer decisions and results
+  if (!(l.v * r.v < 0.0)) {
+    l.v = r.v = 0.0;
+  } else if (std::fabs(l.v) > 2.0 * std::fabs(r.v)) {
+    l.v = -2.0 * r.v;
+  } else if (std::fabs(r.v) > 2.0 * std::fabs(l.v)) {
+    r.v = -2.0 * l.v;
+  }
+}
+
 }  // namespace count
+template <>
+struct PpmByDifferences<count::N64> {
+  static constexpr bool value = true;
+};
 }  // namespace bhac
 
 using namespace bhac;

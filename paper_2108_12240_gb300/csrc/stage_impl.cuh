@@ -602,7 +602,23 @@ __device__ __forceinline__ void strip_edges(int recon, const T* __restrict__ p, 
   T q[S + 4];
 #pragma unroll
   for (int m = 0; m < S + 4; ++m) q[m] = m < n + 4 ? p[(m - 2) * sd] : T(0);
-  if (recon == 0) {
+  if (PpmByDifferences<T>::value && recon == 0) {
+    T d[S + 3];
+#pragma unroll
+    for (int m = 0; m < S + 3; ++m) d[m] = q[m + 1] - q[m];
+    T w = ppm_dev(d[0], d[1], d[2]);
+#pragma unroll
+    for (int m = 0; m < S; ++m) {
+      const T wn = ppm_dev(d[m + 1], d[m + 2], d[m + 3]);
+      T l = w - d[m + 1], r = wn;
+      limit_dev(l, r);
+      if (m < n) {
+        L[m * so] = q[m + 2] + l;
+        R[m * so] = q[m + 2] + r;
+      }
+      w = wn;
+    }
+  } else if (recon == 0) {
     T f[S + 1];
 #pragma unroll
     for (int m = 0; m <= S; ++m) f[m] = ppm_iface(q[m], q[m + 1], q[m + 2], q[m + 3]);
