@@ -92,6 +92,10 @@ template <>
 struct PpmByDifferences<count::N64> {
   static constexpr bool value = true;
 };
+template <>
+struct ShiftedFlux<count::N64> {
+  static constexpr bool value = true;
+};
 }  // namespace bhac
 
 using namespace bhac;
