@@ -177,6 +177,54 @@ BHAC_HD Met<T> load_centre_metric(const R* __restrict__ rec) {
   return m;
 }
 
+// fused multiply-add, and a product rounded on its own: with these an
+// expression's rounding does not depend on which kernel it is compiled into
+template <typename T>
+BHAC_HD T fma_t(T a, T b, T c) { return a * b + c; }
+BHAC_HD double fma_t(double a, double b, double c) { return fma(a, b, c); }
+template <typename T>
+BHAC_HD T mul_rn(T a, T b) {
+  return a * b;
+}
+template <>
+BHAC_HD double mul_rn<double>(double a, double b) {
+#ifdef __CUDA_ARCH__
+  return __dmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+
+constexpr unsigned kHiExp = 0x7FF00000u, kHiOne = 0x00100000u;  // exponent field, exponent unit (high word)
+
+// x / 2, exact for normal results; zeros, non-finite and the smallest normals stay as they are
+template <typename T>
+BHAC_HD T half_t(T x) { return x / T(2); }
+BHAC_HD double half_t(double x) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const bool ok = (hi & kHiExp) - 2u * kHiOne < kHiExp - 2u * kHiOne;
+  return __hiloint2double((int)(ok ? hi - kHiOne : hi), __double2loint(x));
+#else
+  return 0.5 * x;
+#endif
+}
+
+// FP32 companions of an FP64 scalar, for quantities that need seven digits
+// only: truncation (values below the normal FP32 range become 0, above it
+// infinite), exact widening and the hardware reciprocal estimate.
+template <typename T>
+struct LowOf {
+  using type = float;
+};
+__device__ __forceinline__ float low_t(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = hi & kHiExp;
+  const unsigned m = __funnelshift_l(lo, hi, 3) - 0xC0000000u;  // (E - 896) 2^23 + the top 23 significand bits
+  const unsigned r = e < 897u * kHiOne ? 0u : (e > 1150u * kHiOne ? 0x7F800000u : m);
+  return __uint_as_float(r | (hi & 0x80000000u));
+}
+
 // Scalar helpers.  The double/float overloads are the device arithmetic; the
 // flop counter provides overloads for its counting type.
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
@@ -288,7 +336,13 @@ __device__ __forceinline__ double sqrt_t(double x) {
   const unsigned hi = (unsigned)__double2hiint(x);
   unsigned E;
   if ((hi >> 31) || !seed_range(hi, E)) return sqrt(x);
-  return x * rsqrt_pos(x, hi, E);
+  return mul_rn(x, rsqrt_pos(x, hi, E));
+}
+__device__ __forceinline__ double high_t(float x, double) { return widen_f32(x); }
+__device__ __forceinline__ float rcp_low(float x) { return rcp_approx_f32(x); }
+// magnitude within 2^-50 .. 2^50: products of a few such values stay in FP32's range
+__device__ __forceinline__ bool low_range_t(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) - 973u * kHiOne < 100u * kHiOne;
 }
 __device__ __forceinline__ double to_double(double x) { return x; }
 __device__ __forceinline__ double to_double(float x) { return widen_f32(x); }
@@ -544,25 +598,6 @@ template <>
 struct PpmByDifferences<double> {
   static constexpr bool value = true;
 };
-
-template <typename T>
-BHAC_HD T fma_t(T a, T b, T c) { return a * b + c; }
-BHAC_HD double fma_t(double a, double b, double c) { return fma(a, b, c); }
-
-constexpr unsigned kHiExp = 0x7FF00000u, kHiOne = 0x00100000u;  // exponent field, exponent unit (high word)
-
-// x / 2, exact for normal results; zeros, non-finite and the smallest normals stay as they are
-template <typename T>
-BHAC_HD T half_t(T x) { return x / T(2); }
-BHAC_HD double half_t(double x) {
-#ifdef __CUDA_ARCH__
-  const unsigned hi = (unsigned)__double2hiint(x);
-  const bool ok = (hi & kHiExp) - 2u * kHiOne < kHiExp - 2u * kHiOne;
-  return __hiloint2double((int)(ok ? hi - kHiOne : hi), __double2loint(x));
-#else
-  return 0.5 * x;
-#endif
-}
 
 // |a| < |b| by the two words of each (integer pipes; 64-bit masks of a double
 // are turned back into FP64 operations by the compiler)

@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(256) ct_face_kernel(StageArgs a, CtArgs c) {
     if (a.stage == 1)
       c.phi_out[o] = c.phi_in[o] + dt * R;
     else
-      c.phi_out[o] = 0.5 * c.phi_n[o] + 0.5 * (c.phi_in[o] + dt * R);
+      c.phi_out[o] = half_t(c.phi_n[o] + fma_t(dt, R, c.phi_in[o]));
   }
 }
 
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(256) ct_face_level_kernel(StageArgs a, CtArgs 
     if (a.stage == 1)
       c.phi_out[o] = c.phi_in[o] + dt * R;
     else
-      c.phi_out[o] = 0.5 * c.phi_n[o] + 0.5 * (c.phi_in[o] + dt * R);
+      c.phi_out[o] = half_t(c.phi_n[o] + fma_t(dt, R, c.phi_in[o]));
   }
 }
 
@@ -556,13 +556,13 @@ __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) 
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const double un = a.Un[ub + (size_t)v * a.nint];
-      U[v] = a.stage == 1 ? un + dt * rhs[v] : 0.5 * un + 0.5 * (a.U1[ub + (size_t)v * a.nint] + dt * rhs[v]);
+      U[v] = a.stage == 1 ? fma_t(dt, rhs[v], un) : half_t(un + fma_t(dt, rhs[v], a.U1[ub + (size_t)v * a.nint]));
     }
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
       const long long lo = (long long)b * c.g.nfb + ring_index(c.g, d, i, j, k);
       const long long hi = (long long)b * c.g.nfb + ring_index(c.g, d, i + (d == 0), j + (d == 1), k + (d == 2));
-      U[B1 + d] = 0.5 * (c.phi_out[lo] + c.phi_out[hi]);
+      U[B1 + d] = half_t(c.phi_out[lo] + c.phi_out[hi]);
     }
     U[PSI] = 0.0;
     finish_cell<T, DIM, FLAT>(a, geo, b, ci, cg, I1, I2, U, cnt, rate_max);

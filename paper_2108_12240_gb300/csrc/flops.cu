@@ -77,6 +77,11 @@ inline N64 half_t(N64 x) {
   r.v = 0.5 * x.v;
   return r;
 }
+// the FP32 companions: conversions are not counted
+inline N32 low_t(N64 x) { return N32((float)x.v); }
+inline N64 high_t(N32 x, N64) { return N64((double)x.v); }
+inline N32 rcp_low(N32 x) { return rcp_t(x); }
+inline bool low_range_t(N64 x) { return std::fabs(x.v) > 0x1p-50 && std::fabs(x.v) < 0x1p50; }
 inline void limit_dev(N64& l, N64& r) {  // integer decisions and results
   if (!(l.v * r.v < 0.0)) {
     l.v = r.v = 0.0;
@@ -88,6 +93,10 @@ inline void limit_dev(N64& l, N64& r) {  // integer decisions and results
 }
 
 }  // namespace count
+template <>
+struct LowOf<count::N64> {
+  using type = count::N32;
+};
 template <>
 struct PpmByDifferences<count::N64> {
   static constexpr bool value = true;
