@@ -352,7 +352,8 @@ bhac_status bhac_get_diagnostics(bhac_ctx* ctx, long long counts[4]);
 bhac_status bhac_launches_per_step(const bhac_ctx* ctx, int* launches);
 
 /* Kernel launch shape of the stage kernel: tile of tx x ty cells per CTA column
- * (must divide the block), threads per CTA (a multiple of 32, at most 256),
+ * (must divide the block), threads per CTA (a multiple of 32, at most 256; the
+ * library adds two helper warps where the kernel's registers allow),
  * persistent = k > 0 for k CTAs per SM pulling (block, tile) items from a device
  * work counter (0: one CTA per item), and min_ctas = 1, 2 or 3: the register
  * bound the 3-D kernel is compiled for (2 trades a few spilled registers for two

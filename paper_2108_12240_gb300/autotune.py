@@ -19,7 +19,7 @@ SMEM_LIMIT = 226 * 1024
 TWO_CTA_SMEM = 113 * 1024  # per CTA, two CTAs on one SM
 # names the stage kernel's shared-memory design; cached shapes of another
 # design are not reused
-KERNEL_TAG = "edge-staged"
+KERNEL_TAG = "strip-queue"
 
 
 def smem_bytes(tx: int, ty: int, ndim: int, precision: str, producers: int = 0) -> int:
@@ -29,9 +29,11 @@ def smem_bytes(tx: int, ty: int, ndim: int, precision: str, producers: int = 0) 
     if ndim == 3 and producers:
         return 9 * (2 * sfx + 2 * sfy + 3 * sfz) * t
     n = sfx + sfy + 2 * (tx + 2) * ty + 2 * tx * (ty + 2)
-    if ndim == 3:
-        n += 3 * sfz
-    return 9 * n * t
+    if ndim != 3:
+        return 9 * n * t
+    # carried z edges and two z-face planes, a third where it fits beside as many CTAs
+    two, three = 9 * (n + 3 * sfz) * t, 9 * (n + 4 * sfz) * t
+    return three if three <= (TWO_CTA_SMEM if two <= TWO_CTA_SMEM else SMEM_LIMIT) else two
 
 
 def candidates(grid, precision: str, include_ws: bool = False):

@@ -304,19 +304,30 @@ StageArgs base_args(const bhac_ctx* c) {
   return a;
 }
 
-// Shared memory of the stage kernel: face fluxes of one plane (x, y and two
+// Shared memory of the stage kernel: face fluxes of one plane (x, y and zbuf
 // z-face planes), or in the warp-specialised form two planes of x and y faces
 // and three z-face planes.
-size_t stage_smem(const bhac_ctx* c, int tx, int ty, int pwarps) {
+static size_t stage_smem_z(const bhac_ctx* c, int tx, int ty, int pwarps, int zbuf) {
   const size_t tsz = c->mixed ? sizeof(float) : sizeof(double);
   const size_t sFx = (size_t)ty * (tx + 1), sFy = (size_t)(ty + 1) * tx, sFz = (size_t)tx * ty;
   if (c->d.ndim == 3 && pwarps > 0) return NV * (2 * sFx + 2 * sFy + 3 * sFz) * tsz;
   // phased form: face fluxes, edges along x and y (tile plus halo), and in
-  // 3-D two z-face planes and the carried z edges
+  // 3-D zbuf z-face planes and the carried z edges
   const size_t nex = (size_t)(tx + 2) * ty, ney = (size_t)tx * (ty + 2);
   size_t n = sFx + sFy + 2 * nex + 2 * ney;
-  if (c->d.ndim == 3) n += 3 * sFz;
+  if (c->d.ndim == 3) n += (zbuf + 1) * sFz;
   return NV * n * tsz;
+}
+
+// Three z-face planes (the next plane's reconstruction overlaps the cell
+// updates) unless they would not fit, or would cost the second resident CTA.
+int stage_zbuf(const bhac_ctx* c, int tx, int ty, int pwarps) {
+  const size_t lim = stage_smem_z(c, tx, ty, pwarps, 2) <= (size_t)kTwoCtaSmem ? (size_t)kTwoCtaSmem : (size_t)kMaxDynSmem;
+  return stage_smem_z(c, tx, ty, pwarps, 3) <= lim ? 3 : 2;
+}
+
+size_t stage_smem(const bhac_ctx* c, int tx, int ty, int pwarps) {
+  return stage_smem_z(c, tx, ty, pwarps, stage_zbuf(c, tx, ty, pwarps));
 }
 
 bhac_status ghost_fill(bhac_ctx* c, int buf, bool zero_smax) {
@@ -352,6 +363,12 @@ bhac_status ghost_fill(bhac_ctx* c, int buf, bool zero_smax) {
 
 namespace {
 
+// Threads of the phased kernel's CTAs: the size asked for and its helper warps.
+int launch_threads(const bhac_ctx* c) {
+  if (c->split > 0 || c->pwarps > 0) return c->threads;
+  return c->threads + stage_helpers(!c->mixed, c->d.ndim == 3 && c->minb >= 2 ? 2 : 1);
+}
+
 // Z parts per (block, tile) column of the phased 3-D stage kernel.  A fixed
 // choice (bhac_set_zsplit) is used as given.  Otherwise: among the parts that
 // divide nz and leave at least 4 planes, the one that minimises the modelled
@@ -366,8 +383,8 @@ int choose_nzp(const bhac_ctx* c, const StageArgs& a, size_t smem) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int per_sm = c->persistent ? c->persistent
-                                   : (c->mixed ? stage_occupancy_mixed(a, c->threads, smem)
-                                               : stage_occupancy_fp64(a, c->threads, smem));
+                                   : (c->mixed ? stage_occupancy_mixed(a, launch_threads(c), smem)
+                                               : stage_occupancy_fp64(a, launch_threads(c), smem));
   const long long slots = (long long)(nsm > 0 ? nsm : 1) * (per_sm > 0 ? per_sm : 1);
   const long long items = (long long)a.nitems;
   int best = 1;
@@ -404,6 +421,7 @@ bhac_status run_stage(bhac_ctx* c, int stage, double dt) {
     a.Uout = c->U[1 - c->ucur];
   }
   const size_t smem = stage_smem(c, c->tx, c->ty, c->pwarps);
+  a.zbuf = stage_zbuf(c, c->tx, c->ty, c->pwarps);
   if (c->split <= 0 && c->pwarps == 0 && c->d.ndim == 3) {
     // the phased kernel's items may be z parts of (block, tile) columns
     if (c->nzp_eff <= 0) c->nzp_eff = choose_nzp(c, a, smem);
@@ -422,8 +440,8 @@ bhac_status run_stage(bhac_ctx* c, int stage, double dt) {
   }
   cudaError_t e = cudaSuccess;
   if (c->split <= 0) {
-    e = c->mixed ? launch_stage_mixed(a, grid, c->threads, smem, c->st)
-                 : launch_stage_fp64(a, grid, c->threads, smem, c->st);
+    const int threads = launch_threads(c);
+    e = c->mixed ? launch_stage_mixed(a, grid, threads, smem, c->st) : launch_stage_fp64(a, grid, threads, smem, c->st);
   } else {
     // split form: chunk q's face kernel on st, its cell kernel on st2 after it;
     // the face kernel of chunk q + 1 overlaps the cell kernel of chunk q

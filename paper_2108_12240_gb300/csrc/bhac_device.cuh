@@ -43,6 +43,7 @@ struct StageArgs {
   int nblocks, nitems;
   int nzp;               // z parts per (block, tile) item of the phased 3-D kernel (1: whole columns)
   int persistent;
+  int zbuf;              // z-face planes of the phased 3-D kernel in shared memory (2 or 3)
   int minb;              // register bound of the 3-D stage kernel: 1 or 2 CTAs per SM
   int pwarps;            // 3-D: warps that produce face fluxes while the others update cells (0: phased)
   const int* blk;        // nblocks x 4: level, bx, by, bz

@@ -15,6 +15,23 @@ constexpr int kMaxDynSmem = 226 * 1024;
 // per SM, 1 KB of it reserved per resident CTA)
 constexpr int kTwoCtaSmem = 113 * 1024;
 
+// Helper warps: the fused phased stage kernel runs with two warps more than the
+// CTA size asked for.  They have no cells of a 256-cell tile, so they take the
+// next plane's reconstruction from the queue while the other eight invert the
+// current plane's cells, and the 17 warps' worth of x and y faces of a 16x16
+// tile need two rounds instead of three.  Ten warps is what the registers
+// allow: 200 per thread for one CTA per SM, 96 (a few dozen spilled) for two.
+// Measured on the 192x96x96 torus, step with 256, 288, 320, 352 and 384
+// threads: mixed 2.22, 2.02, 1.97, 2.04, 2.04 ms; FP64 with 256, 320, 384 and
+// 512: 11.1, 9.8, 10.0, 10.4 ms.  The FP64 build bound to two CTAs per SM and
+// the split form's face kernels keep 256: they would only spill more.
+constexpr int kHelperThreads = 64;
+constexpr int kStageThreads = 256;
+constexpr int stage_helpers(bool fp64, int minb) {
+  return (minb / 10) % 10 == 0 && (minb % 10 == 1 || (minb % 10 == 2 && !fp64)) ? kHelperThreads : 0;
+}
+constexpr int stage_threads_max(bool fp64, int minb) { return kStageThreads + stage_helpers(fp64, minb); }
+
 // stage kernels (stage_fp64.cu / stage_mixed.cu)
 cudaError_t launch_stage_fp64(const StageArgs& a, int grid, int threads, size_t smem, cudaStream_t st);
 cudaError_t launch_stage_mixed(const StageArgs& a, int grid, int threads, size_t smem, cudaStream_t st);

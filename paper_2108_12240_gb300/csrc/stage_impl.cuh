@@ -276,9 +276,9 @@ BHAC_HD int con2prim_t(const Met<T>& m, const T* U, const T* Pg, size_t ps, T Z0
         c2p_newton_step_t(q, gf, hB, hS2, hBS2, ec, gD, hgD, Z, v2, it >= 1 && it <= 3, dZ, dv2);
       }
       T Zn = Z + dZ, v2n = v2 + dv2;
-      if (!gt0_t(Zn)) Zn = T(0.5) * Z;
-      if (lt0_x(v2n)) v2n = T(0.5) * v2;
-      if (le_x(T(1.0), v2n)) v2n = T(0.5) * (v2 + T(1.0));
+      if (!gt0_t(Zn)) Zn = half_t(Z);
+      if (lt0_x(v2n)) v2n = half_t(v2);
+      if (le_x(T(1.0), v2n)) v2n = half_t(v2 + T(1.0));
       const bool conv = le_x(abs_t(Zn - Z), T(tol) * Zn);
       Z = Zn;
       v2 = v2n;
@@ -1106,7 +1106,8 @@ __device__ __forceinline__ void rk_finish(const StageArgs& a, const LevelGeo& ge
 // The stage kernel.  T: flux arithmetic (double: FP64 form; float: mixed form).
 // Every block of every level is an item of the same launch.
 //
-// Per plane k of the CTA's column, three phases separated by CTA barriers:
+// Per plane k of the CTA's column, three phases, with CTA barriers before and
+// after F:
 //  R  every cell's two reconstructed edges along x (the tile plus one cell on
 //     each x side) and along y (plus one cell on each y side) into shared
 //     memory, by strips of cells of one variable; in 3-D each z column also reconstructs its cell of plane k+1,
@@ -1115,32 +1116,45 @@ __device__ __forceinline__ void rk_finish(const StageArgs& a, const LevelGeo& ge
 //     plane), and keeps plane k+1's high edge for the next plane;
 //  F  the x and y face fluxes from the edges of the two adjacent cells;
 //  C  the cell updates.
+// R's tasks (a warp's worth of z cells or of strips) come from a queue, and
+// with three z-face planes in shared memory no barrier separates C from the
+// next plane's R: a warp that has no cells, or has inverted its own, starts
+// reconstructing while the others still occupy the FP64 unit.  Without the
+// queue and with a barrier there the step of the 192x96x96 torus took 2.29 ms
+// (mixed) against 1.97 with it and the helper warps (launch.h), FP64 11.1
+// against 9.8 ms.
+//
 // Each cell's edges are reconstructed once per direction (up to the one-cell
 // tile halo) instead of once for each of its two faces; the face states are
 // the same numbers as a per-face reconstruction's.
 //
-// Shared memory (T): Fx, Fy, [Fz0, Fz1, EzR in 3-D], ExL, ExR, EyL, EyR.
+// Shared memory (T): Fx, Fy, [three z-face planes and EzR in 3-D], ExL, ExR, EyL, EyR.
 //
 // MINB: the register bound (resident CTAs per SM) in its last digit; + 10: the
 // face kernel of the split form (no inversion code); + 100: the Newton-Krylov
 // inversion in place of the analytic Newton step.
 // ----------------------------------------------------------------------------
 template <typename T, int DIM, bool FLAT, int MINB>
-__global__ void __launch_bounds__(256, MINB % 10) stage_kernel(StageArgs a) {
+__global__ void __launch_bounds__(stage_threads_max(sizeof(T) == 8, MINB), MINB % 10) stage_kernel(StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tx = a.tx, ty = a.ty;
   const int sFx = ty * (tx + 1), sFy = (ty + 1) * tx, sFz = tx * ty;
   const int nex = (tx + 2) * ty, ney = tx * (ty + 2);
   T* Fx = reinterpret_cast<T*>(smem_raw);
   T* Fy = Fx + NV * sFx;
-  T* Fza = Fy + NV * sFy;
-  T* Fzb = Fza + (DIM == 3 ? NV * sFz : 0);
-  T* EzR = Fzb + (DIM == 3 ? NV * sFz : 0);
+  T* Fz = Fy + NV * sFy;  // a.zbuf planes of z faces
+  T* EzR = Fz + (DIM == 3 ? a.zbuf * NV * sFz : 0);
   T* ExL = EzR + (DIM == 3 ? NV * sFz : 0);
   T* ExR = ExL + NV * nex;
   T* EyL = ExR + NV * nex;
   T* EyR = EyL + NV * ney;
   __shared__ int s_item;
+  // next reconstruction task, alternating over the planes this CTA runs: F of
+  // one plane resets the counter of the next
+  __shared__ int s_task[2];
+  if (threadIdx.x < 2) s_task[threadIdx.x] = 0;
+  int par = 0;
+  const int lane = threadIdx.x & 31;
 
   const double dt = stage_dt(a);
   if (a.stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *a.dt_dev = dt;
@@ -1180,8 +1194,10 @@ __global__ void __launch_bounds__(256, MINB % 10) stage_kernel(StageArgs a) {
     const T* Pb = Pb_all + (size_t)b * NV * a.ncell;
     const unsigned cfb = a.nlev > 1 ? a.cf[b] : 0u;
     const bool regs = a.nlev > 1;
-    T* Fz0 = Fza;
-    T* Fz1 = Fzb;
+    T* Fz0 = Fz;
+    T* Fz1 = DIM == 3 ? Fz + NV * sFz : Fz;
+    T* Fz2 = DIM == 3 && a.zbuf == 3 ? Fz1 + NV * sFz : Fz;
+    __syncthreads();
     if (DIM == 3) {
       // bottom face of plane kbeg from the high edge of plane kbeg - 1 and the
       // low edge of plane kbeg; plane kbeg's high edge is kept for the face
@@ -1202,11 +1218,20 @@ __global__ void __launch_bounds__(256, MINB % 10) stage_kernel(StageArgs a) {
         }
         if (regs && kbeg == 0) to_register(a, b, 2, 0, (j + y0) * a.nx + i + x0, Fz0 + t, sFz);
       }
+      __syncthreads();
     }
     for (int k = kbeg; k < kend; ++k) {
       const int kg = k + a.gz;
-      // R: edges (and the z face above plane k)
-      for (int t = threadIdx.x; t < nzc + nlx + nly; t += blockDim.x) {
+      // R: edges (and the z face above plane k), taken by whole warps from a
+      // queue: warps that have no cell of plane k - 1, or are done with it,
+      // are here while the others still invert theirs
+      for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(&s_task[par], 32);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= nzc + nlx + nly) break;
+        t += lane;
+        if (t >= nzc + nlx + nly) continue;
         if (t < nzc) {
           int i, j;
           dtx.split(t, j, i);
@@ -1239,6 +1264,8 @@ __global__ void __launch_bounds__(256, MINB % 10) stage_kernel(StageArgs a) {
       }
       __syncthreads();
       // F: x and y faces
+      par ^= 1;
+      if (threadIdx.x == 0) s_task[par] = 0;
       for (int t = threadIdx.x; t < sFx + sFy; t += blockDim.x) {
         if (t < sFx) {
           int i, j;
@@ -1263,10 +1290,14 @@ __global__ void __launch_bounds__(256, MINB % 10) stage_kernel(StageArgs a) {
       for (int c = threadIdx.x; c < sFz; c += blockDim.x)
         cell_update<T, DIM, FLAT, (MINB % 100 >= 10), (MINB >= 100 ? 1 : 0)>(a, geo, Pb, b, x0, y0, k, c, Fx, Fy, Fz0,
                                                                           Fz1, dt, cfb, cnt, rate_max);
-      __syncthreads();
+      // with three z planes no barrier: the next plane's R touches neither Fx,
+      // Fy nor the two z planes C reads, and the barrier after R is behind
+      // every warp's C
+      if (DIM == 3 && a.zbuf == 2) __syncthreads();
       T* tmp = Fz0;
       Fz0 = Fz1;
-      Fz1 = tmp;
+      Fz1 = Fz2;
+      Fz2 = a.zbuf == 3 ? tmp : Fz0;  // of two planes the third name is the current lower one
     }
     if (!a.persistent) break;
   }
