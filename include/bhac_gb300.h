@@ -356,17 +356,19 @@ bhac_status bhac_launches_per_step(const bhac_ctx* ctx, int* launches);
  * library adds two helper warps where the kernel's registers allow),
  * persistent = k > 0 for k CTAs per SM pulling (block, tile) items from a device
  * work counter (0: one CTA per item), and min_ctas = 1, 2 or 3: the register
- * bound the 3-D kernel is compiled for (2 trades a few spilled registers for two
- * resident CTAs per SM; 3 applies to the face kernel of the split form, see
- * bhac_set_split, and means 2 for the fused kernel), and producer_warps = p > 0 (3-D only, p * 32 < threads)
- * for the warp-specialised form: p warps compute the next plane's face fluxes
+ * bound the kernel is compiled for (2 trades a few spilled registers for two
+ * resident CTAs per SM, and means 1 on 2-D grids in FP64; 3 applies to the face
+ * kernel of the split form, see bhac_set_split, and means 2 for the fused
+ * kernel), and producer_warps = p > 0 (3-D only, p * 32 < threads) for the
+ * warp-specialised form: p warps compute the next plane's face fluxes
  * while the others update the current plane's cells (0: the phased form).
  * tx, ty, threads, min_ctas = 0 keep the current setting.  Results do not
  * depend on the launch shape.  The default after bhac_init_grid: 256 threads,
  * one CTA per item, and the largest of the tiles 32x16, 16x16, 16x8, 8x8
- * that divides the block and fits the shared-memory limit; in the 3-D mixed
- * form the largest of them up to 16x16 that leaves room for two CTAs per SM,
- * with min_ctas = 2. */
+ * that divides the block and fits the shared-memory limit (else the block's
+ * face); in the mixed form the largest of them up to 16x16 that leaves room
+ * for two CTAs per SM, with min_ctas = 2; smaller tiles and CTAs on a grid of
+ * fewer tiles than four fifths of the SMs. */
 bhac_status bhac_set_launch(bhac_ctx* ctx, int tx, int ty, int threads, int persistent, int min_ctas,
                             int producer_warps);
 

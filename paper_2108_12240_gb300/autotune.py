@@ -143,13 +143,34 @@ def cached_or_default(solver, cache_path: str = DEFAULT_CACHE):
         shape = tuple(cache[key]["shape"])
         solver.set_launch(*shape)
         return shape
-    # the library's own default (the rule of bhac_init_grid)
-    nx, ny = solver.grid.nx[0], solver.grid.nx[1]
-    two = solver.grid.ndim == 3 and solver.precision == "mixed"
+    import torch
+    return default_shape(solver.grid, solver.precision,
+                         torch.cuda.get_device_properties(solver.device).multi_processor_count)
+
+
+def default_shape(grid, precision: str, sms: int):
+    """The library's own default (the rule of bhac_init_grid)."""
+    nx, ny, nz = grid.nx
+    mixed = precision == "mixed"
+    limit = TWO_CTA_SMEM if mixed else SMEM_LIMIT
+    shape, threads = [nx, ny], 256
     for tx, ty in ((32, 16), (16, 16), (16, 8), (8, 8)):
-        if two and tx * ty > 256:
+        if mixed and tx * ty > 256:
             continue
-        limit = TWO_CTA_SMEM if two else SMEM_LIMIT
-        if nx % tx == 0 and ny % ty == 0 and smem_bytes(tx, ty, solver.grid.ndim, solver.precision) <= limit:
-            return (tx, ty, 256, 0, 2 if two else 1, 0)
-    return (nx, ny, 256, 0, 1, 0)
+        if nx % tx == 0 and ny % ty == 0 and smem_bytes(tx, ty, grid.ndim, precision) <= limit:
+            shape = [tx, ty]
+            break
+    two = mixed and smem_bytes(*shape, grid.ndim, precision) <= limit
+    parts = 1
+    while grid.ndim == 3 and nz % (2 * parts) == 0 and nz // (2 * parts) >= 4:
+        parts *= 2
+    while 5 * grid.nb * (nx // shape[0]) * (ny // shape[1]) * parts < 4 * sms:
+        k = 0 if shape[0] > shape[1] else 1
+        f = next((f for f in range(2, shape[k]) if shape[k] % f == 0), shape[k])
+        if f <= 1 or shape[0] * shape[1] // f < 16:
+            break
+        shape[k] //= f
+        cells = shape[0] * shape[1]
+        threads = min(256, max(64, -(-cells // 32) * 32))
+        two = two or (mixed and smem_bytes(*shape, grid.ndim, precision) <= limit)
+    return (shape[0], shape[1], threads, 0, 2 if two else 1, 0)

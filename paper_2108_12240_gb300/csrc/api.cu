@@ -366,7 +366,56 @@ namespace {
 // Threads of the phased kernel's CTAs: the size asked for and its helper warps.
 int launch_threads(const bhac_ctx* c) {
   if (c->split > 0 || c->pwarps > 0) return c->threads;
-  return c->threads + stage_helpers(!c->mixed, c->d.ndim == 3 && c->minb >= 2 ? 2 : 1);
+  return c->threads + stage_helpers(!c->mixed, (c->d.ndim == 3 || c->mixed) && c->minb >= 2 ? 2 : 1);
+}
+
+// The launch shape after bhac_init_grid.  The largest of these tiles that
+// divides the block and fits the shared-memory limit, else the whole block
+// face; the mixed form takes tiles of at most 256 cells whose workspace lets
+// two CTAs share an SM, with the two-CTA register bound.  That is the fastest
+// family on every grid large enough to fill the GPU.  A grid whose tiles (times
+// the z parts choose_nzp may cut) are fewer than 4/5 of the SMs gets smaller
+// tiles, halved (or divided by the least factor) along their longer side down
+// to 16 cells: a CTA is bound by its SM's FP64 unit or by latency, so idle SMs
+// cost more than the halo of smaller tiles.  Measured per step: 128x128 shock
+// tube FP64 (64 tiles of 16x16) 155 us, 8x16 and 16x8 101 us, 8x8 105 us;
+// 32x32 cells in 16x16 blocks 153 us, 4x4 tiles 84 us, 4x8 84 us.
+void default_shape(bhac_ctx* c) {
+  static const int tiles[][2] = {{32, 16}, {16, 16}, {16, 8}, {8, 8}};
+  const int* nx = c->d.nx;
+  c->threads = 256;
+  c->minb = 1;
+  c->tx = nx[0];
+  c->ty = nx[1];
+  const size_t limit = c->mixed ? (size_t)kTwoCtaSmem : (size_t)kMaxDynSmem;
+  for (const auto& t : tiles) {
+    if (c->mixed && t[0] * t[1] > 256) continue;
+    if (nx[0] % t[0] == 0 && nx[1] % t[1] == 0 && stage_smem(c, t[0], t[1], 0) <= limit) {
+      c->tx = t[0];
+      c->ty = t[1];
+      break;
+    }
+  }
+  if (c->mixed && stage_smem(c, c->tx, c->ty, 0) <= limit) c->minb = 2;
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  int parts = 1;
+  while (c->d.ndim == 3 && nx[2] % (2 * parts) == 0 && nx[2] / (2 * parts) >= 4) parts *= 2;
+  auto least_factor = [](int n) {
+    for (int f = 2; f * f <= n; ++f)
+      if (n % f == 0) return f;
+    return n;
+  };
+  while (5LL * c->nb * (nx[0] / c->tx) * (nx[1] / c->ty) * parts < 4LL * nsm) {
+    int& side = c->tx > c->ty ? c->tx : c->ty;
+    const int f = least_factor(side);
+    if (f <= 1 || c->tx * c->ty / f < 16) break;
+    side /= f;
+    const int cells = c->tx * c->ty;
+    c->threads = cells >= 256 ? 256 : (cells < 64 ? 64 : (cells + 31) / 32 * 32);
+    if (c->mixed && stage_smem(c, c->tx, c->ty, 0) <= limit) c->minb = 2;
+  }
 }
 
 // Z parts per (block, tile) column of the phased 3-D stage kernel.  A fixed
@@ -677,29 +726,7 @@ bhac_status bhac_init_grid(bhac_ctx** out, const bhac_grid_desc* d, const bhac_b
   c->nef = (long long)C.lv.ef_dst.size();
   c->cur = 0;
   c->ucur = 0;
-  c->threads = 256;
-  // default launch shape: the largest of these tiles that divides the block
-  // and fits the shared-memory limit, else the whole block face.  The 3-D
-  // mixed form takes the largest tile of at most 16 x 16 whose workspace lets
-  // two CTAs share an SM, with the two-CTA register bound: the fastest shape
-  // family on every 3-D grid the autotuner has timed.
-  c->minb = 1;
-  {
-    static const int tiles[][2] = {{32, 16}, {16, 16}, {16, 8}, {8, 8}};
-    c->tx = d->nx[0];
-    c->ty = d->nx[1];
-    const bool two_ctas = d->ndim == 3 && c->mixed;
-    for (const auto& t : tiles) {
-      if (two_ctas && t[0] * t[1] > 256) continue;
-      const size_t limit = two_ctas ? (size_t)kTwoCtaSmem : (size_t)kMaxDynSmem;
-      if (d->nx[0] % t[0] == 0 && d->nx[1] % t[1] == 0 && stage_smem(c, t[0], t[1], 0) <= limit) {
-        c->tx = t[0];
-        c->ty = t[1];
-        if (two_ctas) c->minb = 2;
-        break;
-      }
-    }
-  }
+  default_shape(c);
   c->persistent = 0;
   c->pwarps = 0;
   c->graph = nullptr;

@@ -1641,6 +1641,10 @@ static cudaError_t configure_all_t() {
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = configure_stage_t<T, 2, true, 1>();
   if (e == cudaSuccess) e = configure_stage_t<T, 2, false, 1>();
+  if constexpr (sizeof(T) == 4) {
+    if (e == cudaSuccess) e = configure_stage_t<T, 2, true, 2>();
+    if (e == cudaSuccess) e = configure_stage_t<T, 2, false, 2>();
+  }
   if (e == cudaSuccess) e = configure_stage_t<T, 3, true, 1>();
   if (e == cudaSuccess) e = configure_stage_t<T, 3, false, 1>();
   if (e == cudaSuccess) e = configure_stage_t<T, 3, true, 2>();
@@ -1714,8 +1718,8 @@ static int stage_occupancy_any(const StageArgs& a, int threads, size_t smem) {
                      : (a.flat ? occupancy_t<T, true, 1>(threads, smem) : occupancy_t<T, false, 1>(threads, smem));
 }
 
-// 3-D kernels exist with one or two resident CTAs per SM as the register
-// bound; 2-D grids use the one-CTA form.
+// Kernels exist with one or two resident CTAs per SM as the register bound;
+// 2-D grids in FP64 use the one-CTA form.
 template <typename T>
 static cudaError_t launch_stage_any(const StageArgs& a, int grid, int threads, size_t smem, cudaStream_t st) {
   if (a.split) {
@@ -1740,6 +1744,11 @@ static cudaError_t launch_stage_any(const StageArgs& a, int grid, int threads, s
       return a.flat ? launch_stage_t<T, 3, true, 101>(a, grid, threads, smem, st)
                     : launch_stage_t<T, 3, false, 101>(a, grid, threads, smem, st);
     }
+    if constexpr (sizeof(T) == 4) {
+      if (a.minb >= 2)
+        return a.flat ? launch_stage_t<T, 2, true, 102>(a, grid, threads, smem, st)
+                      : launch_stage_t<T, 2, false, 102>(a, grid, threads, smem, st);
+    }
     return a.flat ? launch_stage_t<T, 2, true, 101>(a, grid, threads, smem, st)
                   : launch_stage_t<T, 2, false, 101>(a, grid, threads, smem, st);
   }
@@ -1749,6 +1758,11 @@ static cudaError_t launch_stage_any(const StageArgs& a, int grid, int threads, s
                     : launch_stage_t<T, 3, false, 2>(a, grid, threads, smem, st);
     return a.flat ? launch_stage_t<T, 3, true, 1>(a, grid, threads, smem, st)
                   : launch_stage_t<T, 3, false, 1>(a, grid, threads, smem, st);
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (a.minb >= 2)
+      return a.flat ? launch_stage_t<T, 2, true, 2>(a, grid, threads, smem, st)
+                    : launch_stage_t<T, 2, false, 2>(a, grid, threads, smem, st);
   }
   return a.flat ? launch_stage_t<T, 2, true, 1>(a, grid, threads, smem, st)
                 : launch_stage_t<T, 2, false, 1>(a, grid, threads, smem, st);
