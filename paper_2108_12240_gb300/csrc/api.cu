@@ -273,6 +273,9 @@ StageArgs base_args(const bhac_ctx* c) {
   a.imex_g = 1.0 - 1.0 / sqrt(2.0);
   a.c2p_gf = (d.gamma_ad - 1.0) / d.gamma_ad;
   a.c2p_v2max = 1.0 - 1.0 / (d.w_max * d.w_max);
+  a.c2p_v2skip = 1.0 - 1.02 / (d.w_max * d.w_max);
+  a.rate_c = 0.0;
+  for (int k = 0; k < d.ndim; ++k) a.rate_c += a.ch * a.idx[k];
   a.rho_fl_c = d.rho_floor;
   a.p_fl_c = d.p_floor;
   a.tab_c = c->tab_c;
@@ -791,6 +794,15 @@ bhac_status bhac_init_grid(bhac_ctx** out, const bhac_grid_desc* d, const bhac_b
   return BHAC_OK;
 }
 
+// what the centre records' CFL rate needs at level l (used with ch >= 1 only)
+static void set_rate_args(const bhac_ctx* c, int l, MetricArgs& M) {
+  const StageArgs a = base_args(c);
+  const double s = (double)(1 << l);
+  M.ndim = a.ndim;
+  M.ch = a.ch;
+  for (int d = 0; d < 3; ++d) M.idx[d] = d < a.ndim ? a.idx[d] * s : a.idx[d];
+}
+
 bhac_status bhac_set_metric(bhac_ctx* c, int kind, double spin, double mass, const double* mks_params) {
   (void)mks_params;
   if (!c) return BHAC_ERR_ARG;
@@ -819,6 +831,7 @@ bhac_status bhac_set_metric(bhac_ctx* c, int kind, double spin, double mass, con
     M.rho_pow = c->d.rho_floor_pow;
     M.p_floor = c->d.p_floor;
     M.p_pow = c->d.p_floor_pow;
+    set_rate_args(c, l, M);
     M.tab_c = c->tab_c + c->toff_c[l] * CREC;
     M.tab_f1 = c->tab_f1 + c->toff_f1[l] * FREC;
     M.tab_f2 = c->tab_f2 + c->toff_f2[l] * FREC;
@@ -847,6 +860,7 @@ bhac_status bhac_set_metric(bhac_ctx* c, int kind, double spin, double mass, con
     M.rho_pow = c->d.rho_floor_pow;
     M.p_floor = c->d.p_floor;
     M.p_pow = c->d.p_floor_pow;
+    set_rate_args(c, l, M);
     M.tab_c = c->te_c + c->teo_c[l] * CREC;
     M.tab_f1 = c->te_f1 + c->teo_f1[l] * FREC;
     M.tab_f2 = c->te_f2 + c->teo_f2[l] * FREC;

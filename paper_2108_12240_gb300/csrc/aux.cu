@@ -220,7 +220,12 @@ __global__ void metric_centre_kernel(MetricArgs M) {
     rec[C_DG22_2] = k.g22.b;
     rec[C_DG33_1] = k.g33.a;
     rec[C_DG33_2] = k.g33.b;
-    for (int q = C_DG33_2 + 1; q < CREC; ++q) rec[q] = 0.0;
+    // sum over active d of (ch alpha sqrt(gamma^dd) + |beta^d|) / dx_d
+    double rate = 0.0;
+    for (int d = 0; d < M.ndim; ++d)
+      rate += (M.ch * rec[C_ACG1 + d] + (d == 0 ? fabs(k.be1.v) : 0.0)) * M.idx[d];
+    rec[C_RATE] = rate;
+    for (int q = C_RATE + 1; q < CREC; ++q) rec[q] = 0.0;
     float* r32 = M.tab_c32 + (size_t)t * CREC;
     for (int q = 0; q < CREC; ++q) r32[q] = (float)rec[q];
   }
@@ -316,9 +321,7 @@ __global__ void init_cons_kernel(StageArgs a, const double* __restrict__ P, doub
       m = load_centre_metric<double>(rec);
       sg = rec[C_SG];
     }
-    Derived<double> s;
-    derive(m, Pc, a.gam_fac, s);
-    cons_of(Pc, s, Uc);
+    cons_direct(m, Pc, a.gam_fac, Uc);
     for (int v = 0; v < NV; ++v) U[((size_t)b * NV + v) * a.nint + ci] = sg * Uc[v];
   }
 }

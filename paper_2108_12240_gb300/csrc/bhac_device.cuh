@@ -28,7 +28,8 @@ enum CRec {
   C_AL = 0, C_BE1, C_G11, C_G13, C_G22, C_G33, C_GI11, C_GI13, C_GI22, C_GI33, C_SG, C_ISG,
   C_ACG1, C_ACG2, C_ACG3, C_RHOFL, C_PFL,
   C_DAL1, C_DAL2, C_DBE1_1, C_DBE1_2, C_DG11_1, C_DG11_2, C_DG13_1, C_DG13_2, C_DG22_1, C_DG22_2,
-  C_DG33_1, C_DG33_2
+  C_DG33_1, C_DG33_2,
+  C_RATE  // ch >= 1: the cell's CFL rate, which then depends on the metric only
 };
 enum FRec { F_AL = 0, F_BE1, F_G11, F_G13, F_G22, F_G33, F_GI11, F_GI13, F_GI22, F_GI33, F_SG, F_ACG };
 
@@ -66,6 +67,8 @@ struct StageArgs {
   int c2p_nk;                // primary inversion: Jacobian-free Newton-Krylov (else analytic Newton)
   double imex_g;             // its gamma = 1 - 1/sqrt(2)
   double wmax, rho_fl_c, p_fl_c;  // constant floors (flat coordinates)
+  double c2p_v2skip;         // below this v^2 a Newton root is clear of the Lorentz-factor ceiling
+  double rate_c;             // flat, ch >= 1: the CFL rate of every level-0 cell
   // state
   const double* P_in;    // FP64 primitives, ghosted
   double* P_out;
@@ -112,6 +115,7 @@ struct LevelGeo {
   const float* tf1_32;
   const float* tf2_32;
   int N1, N2;
+  double scale;  // 2^level
   double idx[3];
   float idx_f[3];
 };
@@ -127,6 +131,7 @@ __host__ __device__ __forceinline__ LevelGeo level_geo(const StageArgs& a, int L
   g.N1 = a.N1l[L];
   g.N2 = a.N2l[L];
   const double s = (double)(1 << L);
+  g.scale = s;
   g.idx[0] = a.idx[0] * s;
   g.idx[1] = a.idx[1] * s;
   g.idx[2] = a.ndim == 3 ? a.idx[2] * s : a.idx[2];
@@ -485,6 +490,30 @@ BHAC_HD void cons_of(const T* P, const Derived<T>& s, T* U) {
   U[CS3] = ZB * s.vl3 - s.Bv * s.Bl3;
   U[CTAU] = Z - P[PRS] + s.Bsq - T(0.5) * s.b2 - U[CD];
   U[B1] = P[B1]; U[B2] = P[B2]; U[B3] = P[B3];
+  U[PSI] = P[PSI];
+}
+
+// The same conserved state in one pass (FP64): D = rho W, with E = rho h W^2 + B^2
+// S_j = (E / W) u_j - (B.v) B_j and tau = E - p_tot - D; 42 FP64 instructions
+// where derive and cons_of take about 60.
+template <typename T>
+BHAC_HD void cons_direct(const Met<T>& m, const T* P, T gam_fac, T* U) {
+  const T u1 = P[U1], u2 = P[U2], u3 = P[U3], B1_ = P[B1], B2_ = P[B2], B3_ = P[B3];
+  const T ul1 = fma_t(m.g11, u1, m.g13 * u3), ul2 = m.g22 * u2, ul3 = fma_t(m.g13, u1, m.g33 * u3);
+  const T Bl1 = fma_t(m.g11, B1_, m.g13 * B3_), Bl2 = m.g22 * B2_, Bl3 = fma_t(m.g13, B1_, m.g33 * B3_);
+  const T W2 = fma_t(u1, ul1, fma_t(u2, ul2, fma_t(u3, ul3, T(1))));
+  const T iW = rsqrt_t(W2);
+  const T Bsq = fma_t(B1_, Bl1, fma_t(B2_, Bl2, B3_ * Bl3));
+  const T Bv = fma_t(B1_, ul1, fma_t(B2_, ul2, B3_ * ul3)) * iW;
+  const T b2 = fma_t(Bsq, iW * iW, Bv * Bv);
+  const T E = fma_t(fma_t(gam_fac, P[PRS], P[RHO]), W2, Bsq);
+  const T c = E * iW;
+  U[CD] = mul_rn(P[RHO], W2 * iW);
+  U[CS1] = fma_t(ul1, c, -(Bl1 * Bv));
+  U[CS2] = fma_t(ul2, c, -(Bl2 * Bv));
+  U[CS3] = fma_t(ul3, c, -(Bl3 * Bv));
+  U[CTAU] = (E - fma_t(T(0.5), b2, P[PRS])) - U[CD];
+  U[B1] = B1_; U[B2] = B2_; U[B3] = B3_;
   U[PSI] = P[PSI];
 }
 

@@ -539,17 +539,27 @@ __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) 
       const T* crec = (sizeof(T) == 8 ? reinterpret_cast<const T*>(geo.tc) : reinterpret_cast<const T*>(geo.tc32)) +
                       (size_t)(I2 * geo.N1 + I1) * CREC;
       const T* Pin = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.P_in) : reinterpret_cast<const T*>(a.P32_in);
-      T Pc[NV], Uc[NV], S[NV];
+      T Pc[NV], S[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) Pc[v] = Pin[(size_t)b * NV * a.ncell + (size_t)v * a.ncell + cg];
       const Met<T> m = load_centre_metric<T>(crec);
-      Derived<T> s;
-      derive(m, Pc, pick<T>(a.gam_fac, a.gam_fac_f), s);
-      cons_of(Pc, s, Uc);
-      sources_of(m, crec, Pc, s, Uc, T(0.0), T(0.0), S);
       const T sg = crec[C_SG];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) rhs[v] += to_double(sg * S[v]);
+      if constexpr (sizeof(T) == 8) {
+        sources_direct(m, crec, Pc, a.gam_fac, T(0.0), T(0.0), S);
+        rhs[CS1] = fma_t(sg, S[0], rhs[CS1]);
+        rhs[CS2] = fma_t(sg, S[1], rhs[CS2]);
+        rhs[CTAU] = fma_t(sg, S[2], rhs[CTAU]);
+      } else {
+        T Uc[NV];
+        Derived<T> s;
+        derive(m, Pc, a.gam_fac_f, s);
+        cons_of(Pc, s, Uc);
+        sources_of(m, crec, Pc, s, Uc, T(0.0), T(0.0), S);
+        // (D, S_3 and B have no source)
+        rhs[CS1] += to_double(sg * S[CS1]);
+        rhs[CS2] += to_double(sg * S[CS2]);
+        rhs[CTAU] += to_double(sg * S[CTAU]);
+      }
     }
     const size_t ub = (size_t)b * NV * a.nint + ci;
     double U[NV];
@@ -565,7 +575,7 @@ __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) 
       U[B1 + d] = half_t(c.phi_out[lo] + c.phi_out[hi]);
     }
     U[PSI] = 0.0;
-    finish_cell<T, DIM, FLAT>(a, geo, b, ci, cg, I1, I2, U, cnt, rate_max);
+    finish_cell<T, DIM, FLAT, (sizeof(T) == 4), 2, true>(a, geo, b, ci, cg, I1, I2, U, cnt, rate_max);
   }
   reduce_outputs(a, cnt, rate_max);
 }

@@ -229,18 +229,22 @@ void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, d
   } else {
     const R* rec = tc + (size_t)(I2 * N1 + I1) * CREC;
     Met<T> m = load_centre_metric<T>(rec);
-    Derived<T> s;
-    T Uc[NV], S_[NV];
-    derive(m, Pc, T(a.gam_fac), s);
-    cons_of(Pc, s, Uc);
-    sources_of(m, rec, Pc, s, Uc, T(a.kappa), T(a.ch * a.ch), S_);
+    T S_[NV];
     sg = crec[C_SG];
     isg = crec[C_ISG];
     rho_fl = crec[C_RHOFL];
     p_fl = crec[C_PFL];
-    if (std::is_same<T, N64>::value) {
-      for (int v = 0; v < NV; ++v) rhs[v] = N64(to_double(rdiv[v])) + N64(sg) * N64(to_double(S_[v]));
+    if constexpr (std::is_same<T, N64>::value) {
+      sources_direct(m, rec, Pc, T(a.gam_fac), T(a.kappa), T(a.ch * a.ch), S_);
+      for (int v = 0; v < NV; ++v) rhs[v] = N64(to_double(rdiv[v]));
+      const int at[4] = {CS1, CS2, CTAU, PSI};
+      for (int q = 0; q < 4; ++q) rhs[at[q]] = fma_t(N64(sg), S_[q], rhs[at[q]]);
     } else {
+      T Uc[NV];
+      Derived<T> s;
+      derive(m, Pc, T(a.gam_fac), s);
+      cons_of(Pc, s, Uc);
+      sources_of(m, rec, Pc, s, Uc, T(a.kappa), T(a.ch * a.ch), S_);
       for (int v = 0; v < NV; ++v) rhs[v] = N64(to_double(rdiv[v] + T(sg) * S_[v]));
     }
   }
@@ -251,7 +255,7 @@ void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, d
   N64 U[NV];
   for (int v = 0; v < NV; ++v) {
     const N64 un = N64(Ub[(size_t)v * a.nint + ci]);
-    U[v] = stage == 1 ? un + N64(dt) * rhs[v] : N64(0.5) * un + N64(0.5) * (un + N64(dt) * rhs[v]);
+    U[v] = stage == 1 ? un + N64(dt) * rhs[v] : half_t(un + (un + N64(dt) * rhs[v]));
   }
   Met<N64> md = a.flat ? flat_metric<N64>() : load_centre_metric<N64>(crec);
   N64 Uu[NV], Pg[NV], Pn[NV];
@@ -279,7 +283,7 @@ void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, d
     c2p_guess<N64>(md, Pg, N64(a.gam_fac), Z0, v20);
   }
   const int st = con2prim_t<N64>(md, Uu, Pg, 1, Z0, v20, N64(rho_fl), N64(p_fl), a.c2p_gf, a.wmax, a.c2p_v2max,
-                                 a.c2p_tol, a.c2p_maxit, a.c2p_nk, Pn);
+                                 a.c2p_v2skip, a.c2p_tol, a.c2p_maxit, a.c2p_nk, Pn);
   if (st >= 2) {
     if (mixed) {
       N32 P32[NV], Uc[NV];
@@ -290,13 +294,13 @@ void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, d
       const N32 sg32 = N32(a.flat ? 1.0f : crec32[C_SG]);
       for (int v = CD; v <= CTAU; ++v) U[v] = N64((double)(sg32 * Uc[v]).v);
     } else {
-      Derived<N64> s;
-      derive(md, Pn, N64(a.gam_fac), s);
-      cons_of(Pn, s, Uu);
+      cons_direct(md, Pn, N64(a.gam_fac), Uu);
       for (int v = 0; v < NV; ++v) U[v] = N64(sg) * Uu[v];
     }
   }
-  if (stage == 2) {
+  // with ch >= 1 the rate is tabulated; below, the light-cone test leaves it
+  // out for nearly every cell of a curved grid
+  if (stage == 2 && a.flat && a.ch < 1.0) {
     N64 acg[3] = {N64(1.0), N64(1.0), N64(1.0)};
     if (!a.flat) {
       acg[0] = N64(crec[C_ACG1]);

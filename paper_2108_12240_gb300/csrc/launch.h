@@ -78,6 +78,8 @@ struct MetricArgs {
   int N1, N2;                   // cells along x1, x2
   int axis_lo, axis_hi;         // polar axis at x2 = low / high boundary
   double rho_floor, rho_pow, p_floor, p_pow;
+  int ndim;                     // CFL rate of the centre records: active dimensions,
+  double ch, idx[3];            // cleaning speed and 1/dx per dimension at this level
   double* tab_c;                // N2 x N1 x CREC
   double* tab_f1;               // N2 x (N1+1) x FREC
   double* tab_f2;               // (N2+1) x N1 x FREC

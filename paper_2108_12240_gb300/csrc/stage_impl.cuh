@@ -61,6 +61,43 @@ BHAC_HD void sources_of(const Met<T>& m, const R* __restrict__ rec, const T* P,
   S[PSI] = -m.al * kappa * P[PSI] - P[PSI] * db11 + ch2 * (B1_ * dal1 + B2_ * dal2);
 }
 
+// The same sources from the primitives in one pass (FP64): with X^i = S^i =
+// E v^i - (B.v) B^i and Y^i = (B.v) v^i + B^i / W^2 the stress is W^ij = X^i v^j
+// - Y^i B^j + p_tot gamma^ij, and tau + D = E - p_tot.  S: the four non-zero
+// sources (S_1, S_2, tau, psi); about 95 FP64 instructions where derive,
+// cons_of and sources_of take about 125.
+template <typename T, typename R>
+BHAC_HD void sources_direct(const Met<T>& m, const R* __restrict__ rec, const T* P, T gam_fac, T kappa, T ch2, T* S) {
+  const T u1 = P[U1], u2 = P[U2], u3 = P[U3], B1_ = P[B1], B2_ = P[B2], B3_ = P[B3];
+  const T ul1 = fma_t(m.g11, u1, m.g13 * u3), ul2 = m.g22 * u2, ul3 = fma_t(m.g13, u1, m.g33 * u3);
+  const T Bl1 = fma_t(m.g11, B1_, m.g13 * B3_), Bl2 = m.g22 * B2_, Bl3 = fma_t(m.g13, B1_, m.g33 * B3_);
+  const T W2 = fma_t(u1, ul1, fma_t(u2, ul2, fma_t(u3, ul3, T(1))));
+  const T iW = rsqrt_t(W2), iW2 = iW * iW;
+  const T Bsq = fma_t(B1_, Bl1, fma_t(B2_, Bl2, B3_ * Bl3));
+  const T Bv = fma_t(B1_, ul1, fma_t(B2_, ul2, B3_ * ul3)) * iW;
+  const T ptot = fma_t(T(0.5), fma_t(Bsq, iW2, Bv * Bv), P[PRS]);
+  const T E = fma_t(fma_t(gam_fac, P[PRS], P[RHO]), W2, Bsq);
+  const T v1 = u1 * iW, v2 = u2 * iW, v3 = u3 * iW, vl1 = ul1 * iW;
+  const T X1 = fma_t(E, v1, -(Bv * B1_)), X2 = fma_t(E, v2, -(Bv * B2_)), X3 = fma_t(E, v3, -(Bv * B3_));
+  const T Y1 = fma_t(Bv, v1, iW2 * B1_), Y2 = fma_t(Bv, v2, iW2 * B2_), Y3 = fma_t(Bv, v3, iW2 * B3_);
+  const T W11 = fma_t(X1, v1, fma_t(-Y1, B1_, ptot * m.gi11));
+  const T W13 = fma_t(X3, v1, fma_t(-Y3, B1_, ptot * m.gi13));
+  const T W22 = fma_t(X2, v2, fma_t(-Y2, B2_, ptot * m.gi22));
+  const T W33 = fma_t(X3, v3, fma_t(-Y3, B3_, ptot * m.gi33));
+  const T W13d = W13 + W13;
+  const T G1 = fma_t(W11, T(rec[C_DG11_1]), fma_t(W13d, T(rec[C_DG13_1]),
+                     fma_t(W22, T(rec[C_DG22_1]), W33 * T(rec[C_DG33_1]))));
+  const T G2 = fma_t(W11, T(rec[C_DG11_2]), fma_t(W13d, T(rec[C_DG13_2]),
+                     fma_t(W22, T(rec[C_DG22_2]), W33 * T(rec[C_DG33_2]))));
+  const T dal1 = T(rec[C_DAL1]), dal2 = T(rec[C_DAL2]), db11 = T(rec[C_DBE1_1]), db12 = T(rec[C_DBE1_2]);
+  const T Et = E - ptot, S1 = fma_t(E, vl1, -(Bv * Bl1)), ha = half_t(m.al);
+  S[0] = fma_t(ha, G1, fma_t(S1, db11, -(Et * dal1)));
+  S[1] = fma_t(ha, G2, fma_t(S1, db12, -(Et * dal2)));
+  const T Wm11 = fma_t(X1, vl1, fma_t(-Y1, Bl1, ptot)), Wm21 = fma_t(X2, vl1, -(Y2 * Bl1));
+  S[2] = fma_t(half_t(m.be1), G1, fma_t(Wm11, db11, fma_t(Wm21, db12, fma_t(-X1, dal1, -(X2 * dal2)))));
+  S[3] = fma_t(-P[PSI], fma_t(m.al, kappa, db11), ch2 * fma_t(B1_, dal1, B2_ * dal2));
+}
+
 // ----------------------------------------------------------------------------
 // Conserved -> primitive inversion (FP64).  Two-dimensional Newton-Raphson in
 // (Z = rho h W^2, v^2) on the momentum and energy equations (Noble et al.
@@ -240,7 +277,8 @@ BHAC_HD void c2p_guess(const Met<T>& m, const T* Pg, T gam_fac, T& Z0, T& v2) {
 // other one).
 template <typename T, int NKM = 2>
 BHAC_HD int con2prim_t(const Met<T>& m, const T* U, const T* Pg, size_t ps, T Z0g, T v2g, T rho_fl, T p_fl,
-                       double gf_d, double wmax_d, double v2max_d, double tol, int maxit, int nk, T* P) {
+                       double gf_d, double wmax_d, double v2max_d, double v2skip_d, double tol, int maxit, int nk,
+                       T* P) {
   const T gf = T(gf_d);
   const T wmax = T(wmax_d);
   const T v2max = T(v2max_d);
@@ -365,7 +403,7 @@ BHAC_HD int con2prim_t(const Met<T>& m, const T* U, const T* Pg, size_t ps, T Z0
   }
   // a Newton root's v^2 is the primitives' 1 - 1/W^2 to within its tolerance,
   // so 2% below the limit the ceiling needs no second look
-  if (status != 0 || !lt_t(v2, T(1.0 - 1.02 * (1.0 - v2max_d)))) {
+  if (status != 0 || !lt_t(v2, T(v2skip_d))) {
     const T gu1 = m.g11 * P[U1] + m.g13 * P[U3];
     const T gu2 = m.g22 * P[U2];
     const T gu3 = m.g13 * P[U1] + m.g33 * P[U3];
@@ -386,7 +424,7 @@ template <int NKM>
 static __device__ __forceinline__ int con2prim(const Met<double>& m, const double* U, const double* Pg, size_t ps,
                                             double Z0, double v20, double rho_fl, double p_fl, const StageArgs& a,
                                             double* P) {
-  return con2prim_t<double, NKM>(m, U, Pg, ps, Z0, v20, rho_fl, p_fl, a.c2p_gf, a.wmax, a.c2p_v2max, a.c2p_tol,
+  return con2prim_t<double, NKM>(m, U, Pg, ps, Z0, v20, rho_fl, p_fl, a.c2p_gf, a.wmax, a.c2p_v2max, a.c2p_v2skip, a.c2p_tol,
                                  a.c2p_maxit, a.c2p_nk, P);
 }
 
@@ -415,6 +453,46 @@ BHAC_HD T cfl_rate_t(const Met<T>& m, const T* acg, const T* P, double gam, doub
     rate = rate + c * T(idx[d]);
   }
   return rate;
+}
+
+// The largest CFL rate so far and a cell's: with ch >= 1 the rate depends on the
+// metric only and is tabulated (C_RATE; flat: one constant per level).  SCREEN
+// (constrained transport, loads, the stand-alone reduction): the signal speeds
+// stay inside the light cone for a physical state and Gamma <= 2, so a cell
+// whose light-cone rate (FP32 records, 1e-5 added for their rounding) is below
+// the largest rate found so far cannot change the maximum, and its three wave
+// speeds (125 FP64 instructions) are not formed.  ``seen``: the bits of a rate
+// already in the result.  Loading, face loading and two mixed steps of
+// constrained transport on 192x96x96 cells went from 8.97 to 7.96 ms with this
+// and cons_direct.  (In the stage kernel the test's registers cost more in
+// spills than it saves: 2.5% of the mixed step.)
+template <int DIM, bool FLAT, bool SCREEN>
+__device__ __forceinline__ void cfl_max(const StageArgs& a, const LevelGeo& geo, const Met<double>& m,
+                                        const double* crec, const float* crec32, const double* P,
+                                        unsigned long long seen, double& rate_max) {
+  double rate;
+  if (a.ch >= 1.0) {
+    rate = FLAT ? a.rate_c * geo.scale : crec[C_RATE];
+  } else {
+    if (SCREEN && !FLAT && a.gam <= 2.0 && gt0_t(P[RHO]) && !lt0_x(P[PRS])) {
+      float b = (crec32[C_ACG1] + fabsf(crec32[C_BE1])) * geo.idx_f[0] + crec32[C_ACG2] * geo.idx_f[1];
+      if (DIM == 3) b += crec32[C_ACG3] * geo.idx_f[2];
+      const double s = __longlong_as_double((long long)seen);
+      if (b * 1.00001f < low_t(lt_t(rate_max, s) ? s : rate_max)) return;
+    }
+    double acg[3] = {1.0, 1.0, 1.0};
+    if (!FLAT) {
+      acg[0] = crec[C_ACG1];
+      acg[1] = crec[C_ACG2];
+      acg[2] = crec[C_ACG3];
+    }
+    rate = cfl_rate_t<double, DIM>(m, acg, P, a.gam, a.gam_fac, a.ch, geo.idx);
+  }
+  rate_max = lt_t(rate_max, rate) ? rate : rate_max;
+}
+// the rate already in the result (0 where none is wanted)
+__device__ __forceinline__ unsigned long long cfl_seen(const StageArgs& a) {
+  return a.ch < 1.0 ? *reinterpret_cast<volatile unsigned long long*>(a.smax_out) : 0ull;
 }
 
 // ----------------------------------------------------------------------------
@@ -869,7 +947,7 @@ __device__ __forceinline__ void to_register(const StageArgs& a, int b, int d, in
 // the Newton starting point comes from the FP32 previous primitives (G32;
 // callers that hold their own FP64 starting point pass G32 = false) and a
 // floored cell's D, S_i, tau are rebuilt in FP32.
-template <typename T, int DIM, bool FLAT, bool G32 = (sizeof(T) == 4), int NKM = 2>
+template <typename T, int DIM, bool FLAT, bool G32 = (sizeof(T) == 4), int NKM = 2, bool SCREEN = false>
 __device__ __forceinline__ void finish_cell(const StageArgs& a, const LevelGeo& geo, int b, int ci, int cg, int I1,
                                             int I2, double U[NV], unsigned cnt[4], double& rate_max) {
   const double* crec = FLAT ? nullptr : geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
@@ -925,9 +1003,7 @@ __device__ __forceinline__ void finish_cell(const StageArgs& a, const LevelGeo& 
 #pragma unroll
       for (int v = CD; v <= CTAU; ++v) U[v] = widen_f32(sg32 * Uc[v]);
     } else {
-      Derived<double> s;
-      derive(md, Pn, a.gam_fac, s);
-      cons_of(Pn, s, Uu);
+      cons_direct(md, Pn, a.gam_fac, Uu);
 #pragma unroll
       for (int v = 0; v < NV; ++v) U[v] = sg * Uu[v];
     }
@@ -945,14 +1021,8 @@ __device__ __forceinline__ void finish_cell(const StageArgs& a, const LevelGeo& 
     for (int v = 0; v < NV; ++v) P3o[(size_t)v * a.ncell] = P32[v];
   }
   if (a.stage == 2) {
-    double acg[3] = {1.0, 1.0, 1.0};
-    if (!FLAT) {
-      acg[0] = crec[C_ACG1];
-      acg[1] = crec[C_ACG2];
-      acg[2] = crec[C_ACG3];
-    }
-    const double rate = cfl_rate_t<double, DIM>(md, acg, Pn, a.gam, a.gam_fac, a.ch, geo.idx);
-    rate_max = lt_t(rate_max, rate) ? rate : rate_max;
+    const float* r32 = FLAT ? nullptr : geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC;
+    cfl_max<DIM, FLAT, SCREEN>(a, geo, md, crec, r32, Pn, SCREEN ? cfl_seen(a) : 0ull, rate_max);
   }
 }
 
@@ -1030,20 +1100,22 @@ __device__ __forceinline__ void cell_update(const StageArgs& a, const LevelGeo& 
       } else {
         m = load_centre_metric<T>(geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC);
       }
-      Derived<T> s;
-      derive(m, Pc, pick<T>(a.gam_fac, a.gam_fac_f), s);
-      cons_of(Pc, s, Uc);
-      if (sizeof(T) == 8)
-        sources_of(m, crec, Pc, s, Uc, pick<T>(kap_x, kap_xf), pick<T>(a.ch * a.ch, a.ch2_f), S);
-      else
+      if constexpr (sizeof(T) == 8) {
+        sources_direct(m, crec, Pc, a.gam_fac, kap_x, a.ch * a.ch, S);
+        const double sg = crec[C_SG];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) rhs[v] = rdiv[v];
+        rhs[CS1] = fma_t(sg, S[0], rhs[CS1]);
+        rhs[CS2] = fma_t(sg, S[1], rhs[CS2]);
+        rhs[CTAU] = fma_t(sg, S[2], rhs[CTAU]);
+        rhs[PSI] = fma_t(sg, S[3], rhs[PSI]);
+      } else {
+        Derived<T> s;
+        derive(m, Pc, pick<T>(a.gam_fac, a.gam_fac_f), s);
+        cons_of(Pc, s, Uc);
         sources_of(m, geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC, Pc, s, Uc, pick<T>(kap_x, kap_xf),
                    pick<T>(a.ch * a.ch, a.ch2_f),
                    S);
-      if (sizeof(T) == 8) {
-        const double sg = crec[C_SG];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) rhs[v] = to_double(rdiv[v]) + sg * to_double(S[v]);
-      } else {
         const T sg = T(geo.tc32[(size_t)(I2 * geo.N1 + I1) * CREC + C_SG]);
 #pragma unroll
         for (int v = 0; v < NV; ++v) rhs[v] = to_double(rdiv[v] + sg * S[v]);
@@ -1531,21 +1603,21 @@ __global__ void __launch_bounds__(256) cfl_kernel(StageArgs a) {
     const int i = ci % a.nx, j = (ci / a.nx) % a.ny, k = ci / (a.nx * a.ny);
     const int cg = ((k + a.gz) * a.Ny + (j + a.gy)) * a.Nx + (i + a.gx);
     const LevelGeo geo = level_geo(a, a.blk[4 * b]);
+    const unsigned long long seen = cfl_seen(a);
     double P[NV];
     const double* Pd = a.P_in + (size_t)b * NV * a.ncell + cg;
 #pragma unroll
     for (int v = 0; v < NV; ++v) P[v] = Pd[(size_t)v * a.ncell];
     Met<double> m = flat_metric<double>();
-    double acg[3] = {1.0, 1.0, 1.0};
+    const double* crec = nullptr;
+    const float* crec32 = nullptr;
     if (!FLAT) {
       const int I1 = a.blk[4 * b + 1] * a.nx + i, I2 = a.blk[4 * b + 2] * a.ny + j;
-      const double* crec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
+      crec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
+      crec32 = geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC;
       m = load_centre_metric<double>(crec);
-      acg[0] = crec[C_ACG1];
-      acg[1] = crec[C_ACG2];
-      acg[2] = crec[C_ACG3];
     }
-    rate_max = fmax(rate_max, cfl_rate_t<double, DIM>(m, acg, P, a.gam, a.gam_fac, a.ch, geo.idx));
+    cfl_max<DIM, FLAT, true>(a, geo, m, crec, crec32, P, seen, rate_max);
   }
   const double w = warp_max_d(rate_max);
   if ((threadIdx.x & 31u) == 0) atomicMax(a.smax_out, (unsigned long long)__double_as_longlong(w));
@@ -1567,6 +1639,7 @@ __global__ void __launch_bounds__(256) load_kernel(StageArgs a, const double* __
     const int i = ci % a.nx, j = (ci / a.nx) % a.ny, k = ci / (a.nx * a.ny);
     const int cg = ((k + a.gz) * a.Ny + (j + a.gy)) * a.Nx + (i + a.gx);
     const LevelGeo geo = level_geo(a, a.blk[4 * b]);
+    const unsigned long long seen = cfl_seen(a);
     double Pc[NV], Uc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -1576,22 +1649,19 @@ __global__ void __launch_bounds__(256) load_kernel(StageArgs a, const double* __
     }
     Met<double> m = flat_metric<double>();
     double sg = 1.0;
-    double acg[3] = {1.0, 1.0, 1.0};
+    const double* rec = nullptr;
+    const float* rec32 = nullptr;
     if (!FLAT) {
       const int I1 = a.blk[4 * b + 1] * a.nx + i, I2 = a.blk[4 * b + 2] * a.ny + j;
-      const double* rec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
+      rec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
+      rec32 = geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC;
       m = load_centre_metric<double>(rec);
       sg = rec[C_SG];
-      acg[0] = rec[C_ACG1];
-      acg[1] = rec[C_ACG2];
-      acg[2] = rec[C_ACG3];
     }
-    Derived<double> s;
-    derive(m, Pc, a.gam_fac, s);
-    cons_of(Pc, s, Uc);
+    cons_direct(m, Pc, a.gam_fac, Uc);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) U[((size_t)b * NV + v) * a.nint + ci] = sg * Uc[v];
-    rate_max = fmax(rate_max, cfl_rate_t<double, DIM>(m, acg, Pc, a.gam, a.gam_fac, a.ch, geo.idx));
+    for (int v = 0; v < NV; ++v) U[((size_t)b * NV + v) * a.nint + ci] = FLAT ? Uc[v] : sg * Uc[v];
+    cfl_max<DIM, FLAT, true>(a, geo, m, rec, rec32, Pc, seen, rate_max);
   }
   const double w = warp_max_d(rate_max);
   if ((threadIdx.x & 31u) == 0) atomicMax(a.smax_out, (unsigned long long)__double_as_longlong(w));
