@@ -274,8 +274,6 @@ StageArgs base_args(const bhac_ctx* c) {
   a.c2p_gf = (d.gamma_ad - 1.0) / d.gamma_ad;
   a.c2p_v2max = 1.0 - 1.0 / (d.w_max * d.w_max);
   a.c2p_v2skip = 1.0 - 1.02 / (d.w_max * d.w_max);
-  a.rate_c = 0.0;
-  for (int k = 0; k < d.ndim; ++k) a.rate_c += a.ch * a.idx[k];
   a.rho_fl_c = d.rho_floor;
   a.p_fl_c = d.p_floor;
   a.tab_c = c->tab_c;
@@ -295,6 +293,12 @@ StageArgs base_args(const bhac_ctx* c) {
     a.toff_c[l] = c->toff_c[l];
     a.toff_f1[l] = c->toff_f1[l];
     a.toff_f2[l] = c->toff_f2[l];
+    a.ratel[l] = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      a.idxl[l][k] = k < d.ndim ? a.idx[k] * (double)(1 << l) : a.idx[k];
+      a.idxl_f[l][k] = (float)a.idxl[l][k];
+      if (k < d.ndim) a.ratel[l] += a.ch * a.idxl[l][k];
+    }
     a.N1l[l] = c->N1g << l;
     a.N2l[l] = c->N2g << l;
   }
@@ -797,10 +801,9 @@ bhac_status bhac_init_grid(bhac_ctx** out, const bhac_grid_desc* d, const bhac_b
 // what the centre records' CFL rate needs at level l (used with ch >= 1 only)
 static void set_rate_args(const bhac_ctx* c, int l, MetricArgs& M) {
   const StageArgs a = base_args(c);
-  const double s = (double)(1 << l);
   M.ndim = a.ndim;
   M.ch = a.ch;
-  for (int d = 0; d < 3; ++d) M.idx[d] = d < a.ndim ? a.idx[d] * s : a.idx[d];
+  for (int d = 0; d < 3; ++d) M.idx[d] = a.idxl[l][d];
 }
 
 bhac_status bhac_set_metric(bhac_ctx* c, int kind, double spin, double mass, const double* mks_params) {

@@ -41,14 +41,15 @@ __global__ void __launch_bounds__(256) ghost_fill_kernel(GhostArgs g) {
       double v[NV];
 #pragma unroll
       for (int q = 0; q < NV; ++q) v[q] = g.P[so + (size_t)q * g.ncell];
+      // signs and clamps on the integer pipes (the FP64 unit issues two lanes a clock)
       if (f & 1u) {
-        v[U2] = -v[U2];
-        v[B2] = -v[B2];
+        v[U2] = __hiloint2double(__double2hiint(v[U2]) ^ (int)0x80000000, __double2loint(v[U2]));
+        v[B2] = __hiloint2double(__double2hiint(v[B2]) ^ (int)0x80000000, __double2loint(v[B2]));
       }
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        if ((f >> (1 + 2 * d)) & 1u) v[U1 + d] = v[U1 + d] > 0.0 ? 0.0 : v[U1 + d];
-        if ((f >> (2 + 2 * d)) & 1u) v[U1 + d] = v[U1 + d] < 0.0 ? 0.0 : v[U1 + d];
+        if ((f >> (1 + 2 * d)) & 1u) v[U1 + d] = gt0_t(v[U1 + d]) ? 0.0 : v[U1 + d];
+        if ((f >> (2 + 2 * d)) & 1u) v[U1 + d] = lt0_x(v[U1 + d]) ? 0.0 : v[U1 + d];
       }
 #pragma unroll
       for (int q = 0; q < NV; ++q) g.P[dout + (size_t)q * g.ncell] = v[q];

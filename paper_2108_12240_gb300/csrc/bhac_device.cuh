@@ -68,7 +68,6 @@ struct StageArgs {
   double imex_g;             // its gamma = 1 - 1/sqrt(2)
   double wmax, rho_fl_c, p_fl_c;  // constant floors (flat coordinates)
   double c2p_v2skip;         // below this v^2 a Newton root is clear of the Lorentz-factor ceiling
-  double rate_c;             // flat, ch >= 1: the CFL rate of every level-0 cell
   // state
   const double* P_in;    // FP64 primitives, ghosted
   double* P_out;
@@ -95,6 +94,11 @@ struct StageArgs {
   int nlev;
   long long toff_c[MAXLEV], toff_f1[MAXLEV], toff_f2[MAXLEV];
   int N1l[MAXLEV], N2l[MAXLEV];
+  // per level 1/dx (its FP32 copy) and, flat with ch >= 1, the CFL rate of
+  // every cell: tabulated, since the FP64 unit also does the conversions
+  double idxl[MAXLEV][3];
+  float idxl_f[MAXLEV][3];
+  double ratel[MAXLEV];
   // coarse-fine faces: per block, bit 2d+s marks a face bordering finer blocks
   // (its adjacent cells are finished by the reflux pass); per block x 6 the
   // element offset of the face's flux register, or -1
@@ -115,7 +119,7 @@ struct LevelGeo {
   const float* tf1_32;
   const float* tf2_32;
   int N1, N2;
-  double scale;  // 2^level
+  double rate;
   double idx[3];
   float idx_f[3];
 };
@@ -130,12 +134,11 @@ __host__ __device__ __forceinline__ LevelGeo level_geo(const StageArgs& a, int L
   g.tf2_32 = a.tab_f2_32 ? a.tab_f2_32 + a.toff_f2[L] * FREC : nullptr;
   g.N1 = a.N1l[L];
   g.N2 = a.N2l[L];
-  const double s = (double)(1 << L);
-  g.scale = s;
-  g.idx[0] = a.idx[0] * s;
-  g.idx[1] = a.idx[1] * s;
-  g.idx[2] = a.ndim == 3 ? a.idx[2] * s : a.idx[2];
-  for (int d = 0; d < 3; ++d) g.idx_f[d] = (float)g.idx[d];
+  g.rate = a.ratel[L];
+  for (int d = 0; d < 3; ++d) {
+    g.idx[d] = a.idxl[L][d];
+    g.idx_f[d] = a.idxl_f[L][d];
+  }
   return g;
 }
 

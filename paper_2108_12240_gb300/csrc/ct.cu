@@ -412,7 +412,7 @@ __device__ __forceinline__ double emf2(const CtArgs& c, int b, int i, int j, int
 // d_t Phi = -curl E and the stage combination, one thread per owned face.
 template <int DIM>
 __global__ void __launch_bounds__(256) ct_face_kernel(StageArgs a, CtArgs c) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   const unsigned n = (unsigned)a.nblocks * (unsigned)c.g.nown_b;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int b = (int)(t / (unsigned)c.g.nown_b);
@@ -474,7 +474,7 @@ __device__ __forceinline__ double emf_at(const CtArgs& c, int b, int e, int i, i
 // spacing, and the stage combination, one thread per owned face.
 template <int DIM>
 __global__ void __launch_bounds__(256) ct_face_level_kernel(StageArgs a, CtArgs c) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   const unsigned n = (unsigned)a.nblocks * (unsigned)c.g.nown_b;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int b = (int)(t / (unsigned)c.g.nown_b);
@@ -487,8 +487,7 @@ __global__ void __launch_bounds__(256) ct_face_level_kernel(StageArgs a, CtArgs 
       c.phi_out[o] = 0.0;  // sqrt(gamma) = 0 on the axis
       continue;
     }
-    const double s = (double)(1 << L);
-    const double ix = a.idx[0] * s, iy = a.idx[1] * s, iz = DIM == 3 ? a.idx[2] * s : a.idx[2];
+    const double ix = a.idxl[L][0], iy = a.idxl[L][1], iz = a.idxl[L][2];
     double R;
     if (d == 0) {
       R = -(emf_at(c, b, 2, i, j + 1, k) - emf_at(c, b, 2, i, j, k)) * iy;
@@ -514,7 +513,7 @@ __global__ void __launch_bounds__(256) ct_face_level_kernel(StageArgs a, CtArgs 
 // few spilled values; the mixed form's stage 2.5% faster than at one CTA).
 template <typename T, int DIM, bool FLAT>
 __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   if (a.stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *a.dt_dev = dt;
   unsigned cnt[4] = {0u, 0u, 0u, 0u};
   double rate_max = 0.0;

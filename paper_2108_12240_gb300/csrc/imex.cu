@@ -11,7 +11,7 @@ namespace bhac {
 namespace {
 
 __global__ void __launch_bounds__(256) imex_first_stage_kernel(StageArgs a, double* P, float* P32) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   const long long n = (long long)a.nblocks * a.nint;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(t / a.nint);

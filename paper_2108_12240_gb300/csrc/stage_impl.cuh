@@ -18,10 +18,16 @@
 
 namespace bhac {
 
+// Largest of the warp's values (none negative, as rates are): their bits order
+// like the values, so the FP64 unit is left out.
 __device__ __forceinline__ double warp_max_d(double v) {
+  unsigned long long b = (unsigned long long)__double_as_longlong(v);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, b, o);
+    b = x > b ? x : b;
+  }
+  return __longlong_as_double((long long)b);
 }
 
 // ----------------------------------------------------------------------------
@@ -472,7 +478,7 @@ __device__ __forceinline__ void cfl_max(const StageArgs& a, const LevelGeo& geo,
                                         unsigned long long seen, double& rate_max) {
   double rate;
   if (a.ch >= 1.0) {
-    rate = FLAT ? a.rate_c * geo.scale : crec[C_RATE];
+    rate = FLAT ? geo.rate : crec[C_RATE];
   } else {
     if (SCREEN && !FLAT && a.gam <= 2.0 && gt0_t(P[RHO]) && !lt0_x(P[PRS])) {
       float b = (crec32[C_ACG1] + fabsf(crec32[C_BE1])) * geo.idx_f[0] + crec32[C_ACG2] * geo.idx_f[1];
@@ -1032,6 +1038,15 @@ __device__ __forceinline__ double stage_dt(const StageArgs& a) {
   return *a.dt_dev;
 }
 
+// The same for a whole CTA, the division done once: a thread's own would cost
+// as many FP64 instructions as a tenth of a cell's inversion.
+__device__ __forceinline__ double block_dt(const StageArgs& a) {
+  __shared__ double s_dt;
+  if (threadIdx.x == 0) s_dt = stage_dt(a);
+  __syncthreads();
+  return s_dt;
+}
+
 __device__ __forceinline__ void reduce_outputs(const StageArgs& a, const unsigned cnt[4], double rate_max) {
   const unsigned lane = threadIdx.x & 31u;
 #pragma unroll
@@ -1228,7 +1243,7 @@ __global__ void __launch_bounds__(stage_threads_max(sizeof(T) == 8, MINB), MINB 
   int par = 0;
   const int lane = threadIdx.x & 31;
 
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   if (a.stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *a.dt_dev = dt;
 
   const T* Pb_all = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.P_in) : reinterpret_cast<const T*>(a.P32_in);
@@ -1450,7 +1465,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel_ws(StageArgs a) {
   for (int q = 0; q < 3; ++q) FzB[q] = base + 2 * NV * (sFx + sFy) + q * NV * sFz;
   __shared__ int s_item;
 
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   if (a.stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *a.dt_dev = dt;
   const T* Pb_all = sizeof(T) == 8 ? reinterpret_cast<const T*>(a.P_in) : reinterpret_cast<const T*>(a.P32_in);
   const int nthr = blockDim.x, nprod = a.pwarps * 32, ncons = nthr - nprod;
@@ -1506,7 +1521,7 @@ __global__ void __launch_bounds__(256, MINB) stage_kernel_ws(StageArgs a) {
 // rk_finish (the same arithmetic as the fused kernel).
 template <typename T, int DIM, bool FLAT>
 __global__ void __launch_bounds__(256) cell_kernel(StageArgs a) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   unsigned cnt[4] = {0u, 0u, 0u, 0u};
   double rate_max = 0.0;
   const int tx = a.tx, ty = a.ty, ntile = a.ntx * a.nty;
@@ -1553,7 +1568,7 @@ static cudaError_t launch_cells_any(const StageArgs& a, int grid, cudaStream_t s
 // and 1/2 in stage 2), then is inverted like every other cell.
 template <typename T, int DIM, bool FLAT>
 __global__ void __launch_bounds__(128) reflux_kernel(StageArgs a) {
-  const double dt = stage_dt(a);
+  const double dt = block_dt(a);
   const double f = a.stage == 1 ? 1.0 : 0.5;
   unsigned cnt[4] = {0u, 0u, 0u, 0u};
   double rate_max = 0.0;
