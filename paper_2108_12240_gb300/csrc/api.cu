@@ -891,13 +891,14 @@ bhac_status bhac_set_prims(bhac_ctx* c, const double* prims, int on_device) {
   StageArgs a = base_args(c);
   // one pass: ghosted primitives, conserved state and the CFL rate
   cudaError_t e = cudaMemsetAsync(c->smax, 0, sizeof(unsigned long long), c->st);
+  if (c->ct) a.smax_out = nullptr;  // the faces that follow change the field: no rate yet
   if (e == cudaSuccess) e = launch_load(a, src, c->P[0], c->P32[0], c->U[0], c->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, (size_t)c->nb * c->nint, c->st);
   if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return BHAC_ERR_CUDA;
   c->prims_ok = true;
   c->cfl_ok = false;
-  c->cfl_fresh = true;
+  c->cfl_fresh = !c->ct;
   c->faces_ok = false;
   c->pcur = 0;
   return BHAC_OK;
@@ -940,13 +941,14 @@ bhac_status bhac_set_prims_host_async(bhac_ctx* c, const double* host_prims) {
   // one pass: ghosted primitives, conserved state and the CFL rate; then the
   // staging buffer is free for the next load
   e = cudaMemsetAsync(c->smax, 0, sizeof(unsigned long long), c->st);
+  if (c->ct) a.smax_out = nullptr;
   if (e == cudaSuccess) e = launch_load(a, c->scratch, c->P[0], c->P32[0], c->U[0], c->st);
   if (e == cudaSuccess) e = cudaEventRecord(c->ev_scat, c->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, (size_t)c->nb * c->nint, c->st);
   if (e != cudaSuccess) return BHAC_ERR_CUDA;
   c->prims_ok = true;
   c->cfl_ok = false;
-  c->cfl_fresh = true;
+  c->cfl_fresh = !c->ct;
   c->faces_ok = false;
   c->pcur = 0;
   return BHAC_OK;
@@ -1209,14 +1211,15 @@ bhac_status bhac_set_faces(bhac_ctx* c, const double* faces, int on_device) {
   StageArgs a = base_args(c);
   CtArgs t = ct_args(c);
   cudaError_t e = launch_ct_copy_faces(a, c->ctg, src, c->phi[0], 1, c->st);
-  // the cell field of the loaded primitives from the faces, then U
-  if (e == cudaSuccess) e = launch_ct_cell_field(a, t, c->P[c->cur], c->mixed ? c->P32[c->cur] : nullptr, c->st);
-  if (e == cudaSuccess) e = launch_init_cons(a, c->P[c->cur], c->U[c->ucur], c->st);
+  // the cell field of the loaded primitives from the faces, U and the CFL rate
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->smax, 0, sizeof(unsigned long long), c->st);
+  if (e == cudaSuccess)
+    e = launch_ct_load(a, t, c->P[c->cur], c->mixed ? c->P32[c->cur] : nullptr, c->U[c->ucur], c->st);
   if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return BHAC_ERR_CUDA;
   c->faces_ok = true;
   c->cfl_ok = false;
-  c->cfl_fresh = false;  // the cell field now comes from the faces
+  c->cfl_fresh = true;
   return BHAC_OK;
 }
 

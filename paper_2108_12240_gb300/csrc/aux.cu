@@ -285,7 +285,7 @@ cudaError_t launch_metric_tables(const MetricArgs& M, cudaStream_t st) {
 }
 
 // ----------------------------------------------------------------------------
-// Interior <-> ghosted copies and the conserved state of given primitives.
+// Read-out of the interior primitives.
 // ----------------------------------------------------------------------------
 __device__ __forceinline__ void interior_coords(const StageArgs& a, long long t, int& b, int& ci, int& cg, int& i,
                                                 int& j) {
@@ -306,34 +306,8 @@ __global__ void gather_kernel(StageArgs a, const double* __restrict__ P, double*
   }
 }
 
-__global__ void init_cons_kernel(StageArgs a, const double* __restrict__ P, double* U) {
-  const long long n = (long long)a.nblocks * a.nint;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    int b, ci, cg, i, j;
-    interior_coords(a, t, b, ci, cg, i, j);
-    double Pc[NV], Uc[NV];
-    for (int v = 0; v < NV; ++v) Pc[v] = P[((size_t)b * NV + v) * a.ncell + cg];
-    Met<double> m = flat_metric<double>();
-    double sg = 1.0;
-    if (!a.flat) {
-      const LevelGeo geo = level_geo(a, a.blk[4 * b]);
-      const int I1 = a.blk[4 * b + 1] * a.nx + i, I2 = a.blk[4 * b + 2] * a.ny + j;
-      const double* rec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
-      m = load_centre_metric<double>(rec);
-      sg = rec[C_SG];
-    }
-    cons_direct(m, Pc, a.gam_fac, Uc);
-    for (int v = 0; v < NV; ++v) U[((size_t)b * NV + v) * a.nint + ci] = sg * Uc[v];
-  }
-}
-
 cudaError_t launch_gather_interior(const StageArgs& a, const double* P, double* dst, cudaStream_t st) {
   gather_kernel<<<grid_for((long long)a.nblocks * a.nint, 256), 256, 0, st>>>(a, P, dst);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_init_cons(const StageArgs& a, const double* P, double* U, cudaStream_t st) {
-  init_cons_kernel<<<grid_for((long long)a.nblocks * a.nint, 256), 256, 0, st>>>(a, P, U);
   return cudaGetLastError();
 }
 

@@ -370,16 +370,21 @@ __device__ __forceinline__ void ct_one_face(const StageArgs& a, const CtArgs& c,
   for (int v = 0; v < NV; ++v) c.xf[o + v * c.g.nfd[D]] = to_double(F[v]);
 }
 
-// Fluxes through every face of every block and its ring, one thread per face.
+// Fluxes through every face of every block and its ring, one thread per face,
+// all faces of direction 0 first, then 1, then 2: the three directions' code
+// together is larger than an SM's instruction cache (block by block instead:
+// 605 against 535 us for 7.1 M faces in FP32, with 3.5 of 12 stall cycles per
+// instruction waiting for instructions).
 template <typename T, bool FLAT>
 __global__ void __launch_bounds__(256) ct_flux_kernel(StageArgs a, CtArgs c) {
   // 32-bit index arithmetic: bhac_init_grid keeps blocks x ring-extended faces below 2^31
+  const unsigned n0 = (unsigned)a.nblocks * (unsigned)c.g.nfd[0], n1 = n0 + (unsigned)a.nblocks * (unsigned)c.g.nfd[1];
   const unsigned n = (unsigned)a.nblocks * (unsigned)c.g.nfb;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const int b = (int)(t / (unsigned)c.g.nfb);
-    const int r = (int)(t - (unsigned)b * (unsigned)c.g.nfb);
-    const int d = (c.g.ndim == 3 && r >= c.g.foff[2]) ? 2 : (r >= c.g.foff[1] ? 1 : 0);
-    const int q = r - (int)c.g.foff[d];
+    const int d = t < n0 ? 0 : (t < n1 ? 1 : 2);
+    const unsigned u = d == 0 ? t : (d == 1 ? t - n0 : t - n1), nf = (unsigned)c.g.nfd[d];
+    const int b = (int)(u / nf);
+    const int q = (int)(u - (unsigned)b * nf);
     const int e0 = c.g.fe[d][0], e1 = c.g.fe[d][1];
     const int i = q % e0 - c.g.fo[d][0];
     const int j = (q / e0) % e1 - c.g.fo[d][1];
@@ -393,19 +398,21 @@ __global__ void __launch_bounds__(256) ct_flux_kernel(StageArgs a, CtArgs c) {
   }
 }
 
-// Edge EMFs: E_3 at (i-1/2, j-1/2) of cell layer k, E_1 at (j-1/2, k-1/2) of
-// column i, E_2 at (k-1/2, i-1/2) of row j.
-__device__ __forceinline__ double emf3(const CtArgs& c, int b, int i, int j, int k) {
-  return 0.25 * (xf_at(c, b, 1, B1, i, j, k) + xf_at(c, b, 1, B1, i - 1, j, k) - xf_at(c, b, 0, B2, i, j, k) -
-                 xf_at(c, b, 0, B2, i, j - 1, k));
+// Four times the edge EMFs: E_3 at (i-1/2, j-1/2) of cell layer k, E_1 at
+// (j-1/2, k-1/2) of column i, E_2 at (k-1/2, i-1/2) of row j.  (The quarter is
+// exact wherever it is applied; the face update, bound by its 20 FP64
+// instructions per face, applies it to 1/dx and needs 16.)
+__device__ __forceinline__ double emf3x4(const CtArgs& c, int b, int i, int j, int k) {
+  return xf_at(c, b, 1, B1, i, j, k) + xf_at(c, b, 1, B1, i - 1, j, k) - xf_at(c, b, 0, B2, i, j, k) -
+         xf_at(c, b, 0, B2, i, j - 1, k);
 }
-__device__ __forceinline__ double emf1(const CtArgs& c, int b, int i, int j, int k) {
-  return 0.25 * (xf_at(c, b, 2, B2, i, j, k) + xf_at(c, b, 2, B2, i, j - 1, k) - xf_at(c, b, 1, B3, i, j, k) -
-                 xf_at(c, b, 1, B3, i, j, k - 1));
+__device__ __forceinline__ double emf1x4(const CtArgs& c, int b, int i, int j, int k) {
+  return xf_at(c, b, 2, B2, i, j, k) + xf_at(c, b, 2, B2, i, j - 1, k) - xf_at(c, b, 1, B3, i, j, k) -
+         xf_at(c, b, 1, B3, i, j, k - 1);
 }
-__device__ __forceinline__ double emf2(const CtArgs& c, int b, int i, int j, int k) {
-  return 0.25 * (xf_at(c, b, 0, B3, i, j, k) + xf_at(c, b, 0, B3, i, j, k - 1) - xf_at(c, b, 2, B1, i, j, k) -
-                 xf_at(c, b, 2, B1, i - 1, j, k));
+__device__ __forceinline__ double emf2x4(const CtArgs& c, int b, int i, int j, int k) {
+  return xf_at(c, b, 0, B3, i, j, k) + xf_at(c, b, 0, B3, i, j, k - 1) - xf_at(c, b, 2, B1, i, j, k) -
+         xf_at(c, b, 2, B1, i - 1, j, k);
 }
 
 
@@ -424,16 +431,17 @@ __global__ void __launch_bounds__(256) ct_face_kernel(StageArgs a, CtArgs c) {
       c.phi_out[o] = 0.0;  // sqrt(gamma) = 0 on the axis
       continue;
     }
+    const double qx = 0.25 * a.idx[0], qy = 0.25 * a.idx[1], qz = 0.25 * a.idx[2];
     double R;
     if (d == 0) {
-      R = -(emf3(c, b, i, j + 1, k) - emf3(c, b, i, j, k)) * a.idx[1];
-      if (DIM == 3) R += (emf2(c, b, i, j, k + 1) - emf2(c, b, i, j, k)) * a.idx[2];
+      R = -(emf3x4(c, b, i, j + 1, k) - emf3x4(c, b, i, j, k)) * qy;
+      if (DIM == 3) R += (emf2x4(c, b, i, j, k + 1) - emf2x4(c, b, i, j, k)) * qz;
     } else if (d == 1) {
-      R = (emf3(c, b, i + 1, j, k) - emf3(c, b, i, j, k)) * a.idx[0];
-      if (DIM == 3) R -= (emf1(c, b, i, j, k + 1) - emf1(c, b, i, j, k)) * a.idx[2];
+      R = (emf3x4(c, b, i + 1, j, k) - emf3x4(c, b, i, j, k)) * qx;
+      if (DIM == 3) R -= (emf1x4(c, b, i, j, k + 1) - emf1x4(c, b, i, j, k)) * qz;
     } else {
-      R = -(emf2(c, b, i + 1, j, k) - emf2(c, b, i, j, k)) * a.idx[0] +
-          (emf1(c, b, i, j + 1, k) - emf1(c, b, i, j, k)) * a.idx[1];
+      R = -(emf2x4(c, b, i + 1, j, k) - emf2x4(c, b, i, j, k)) * qx +
+          (emf1x4(c, b, i, j + 1, k) - emf1x4(c, b, i, j, k)) * qy;
     }
     if (a.stage == 1)
       c.phi_out[o] = c.phi_in[o] + dt * R;
@@ -451,7 +459,7 @@ __global__ void __launch_bounds__(256) ct_emf_kernel(StageArgs a, CtArgs c) {
     const int e = r >= c.g.eoff[2] ? 2 : (r >= c.g.eoff[1] ? 1 : 0);
     const int q = r - (int)c.g.eoff[e];
     const int i = q % c.g.ee[e][0], j = (q / c.g.ee[e][0]) % c.g.ee[e][1], k = q / (c.g.ee[e][0] * c.g.ee[e][1]);
-    c.emf[t] = e == 0 ? emf1(c, b, i, j, k) : (e == 1 ? emf2(c, b, i, j, k) : emf3(c, b, i, j, k));
+    c.emf[t] = 0.25 * (e == 0 ? emf1x4(c, b, i, j, k) : (e == 1 ? emf2x4(c, b, i, j, k) : emf3x4(c, b, i, j, k)));
   }
 }
 
@@ -579,41 +587,68 @@ __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) 
   reduce_outputs(a, cnt, rate_max);
 }
 
-// The cell field of the loaded state from its faces.
-template <int DIM>
-__global__ void __launch_bounds__(256) ct_cell_field_kernel(StageArgs a, CtArgs c, double* P, float* P32) {
-  const long long n = (long long)a.nblocks * a.nint;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / a.nint);
-    const int ci = (int)(t - (long long)b * a.nint);
+// After a face load, in one pass over the interior cells (three passes, one of
+// them for the rate, took 565 us on 1.8 M cells): the cell field of the
+// loaded primitives from its faces (psi = 0), the conserved state, and the CFL
+// rate of the state reduced into smax_out.
+template <int DIM, bool FLAT>
+__global__ void __launch_bounds__(256) ct_load_kernel(StageArgs a, CtArgs c, double* P, float* P32, double* U) {
+  double rate_max = 0.0;
+  const unsigned n = (unsigned)a.nblocks * (unsigned)a.nint;
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const int b = (int)(t / (unsigned)a.nint);
+    const int ci = (int)(t - (unsigned)b * (unsigned)a.nint);
     const int i = ci % a.nx, j = (ci / a.nx) % a.ny, k = ci / (a.nx * a.ny);
     const int cg = ((k + a.gz) * a.Ny + (j + a.gy)) * a.Nx + (i + a.gx);
-    double sg = 1.0;
-    if (!a.flat) {
-      const int L = a.blk[4 * b];
+    const LevelGeo geo = level_geo(a, a.blk[4 * b]);
+    const unsigned long long seen = cfl_seen(a);
+    Met<double> m = flat_metric<double>();
+    const double* rec = nullptr;
+    const float* rec32 = nullptr;
+    double sg = 1.0, isg = 1.0;
+    if (!FLAT) {
       const int I1 = a.blk[4 * b + 1] * a.nx + i, I2 = a.blk[4 * b + 2] * a.ny + j;
-      sg = a.tab_c[((size_t)a.toff_c[L] + (size_t)I2 * a.N1l[L] + I1) * CREC + C_SG];
+      rec = geo.tc + (size_t)(I2 * geo.N1 + I1) * CREC;
+      rec32 = geo.tc32 + (size_t)(I2 * geo.N1 + I1) * CREC;
+      m = load_centre_metric<double>(rec);
+      sg = rec[C_SG];
+      isg = rec[C_ISG];
     }
-    double* Pc = P + (size_t)b * NV * a.ncell + cg;
+    double* Pb = P + (size_t)b * NV * a.ncell + cg;
+    double Pc[NV], Uc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Pc[v] = Pb[(size_t)v * a.ncell];
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
       const long long lo = (long long)b * c.g.nfb + ring_index(c.g, d, i, j, k);
       const long long hi = (long long)b * c.g.nfb + ring_index(c.g, d, i + (d == 0), j + (d == 1), k + (d == 2));
-      Pc[(size_t)(B1 + d) * a.ncell] = 0.5 * (c.phi_in[lo] + c.phi_in[hi]) / sg;
-      if (P32) P32[(size_t)b * NV * a.ncell + cg + (size_t)(B1 + d) * a.ncell] = narrow_f64(Pc[(size_t)(B1 + d) * a.ncell]);
+      // the quotient by sqrt(gamma): the product with its reciprocal and one correction
+      const double x = half_t(c.phi_in[lo] + c.phi_in[hi]), q = x * isg;
+      Pc[B1 + d] = fma(fma(-q, sg, x), isg, q);
     }
-    Pc[(size_t)PSI * a.ncell] = 0.0;
-    if (P32) P32[(size_t)b * NV * a.ncell + cg + (size_t)PSI * a.ncell] = 0.0f;
+    Pc[PSI] = 0.0;
+    cons_direct(m, Pc, a.gam_fac, Uc);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      U[((size_t)b * NV + v) * a.nint + ci] = FLAT ? Uc[v] : sg * Uc[v];
+      if ((v >= B1 && v < B1 + DIM) || v == PSI) {
+        Pb[(size_t)v * a.ncell] = Pc[v];
+        if (P32) P32[(size_t)b * NV * a.ncell + cg + (size_t)v * a.ncell] = narrow_f64(Pc[v]);
+      }
+    }
+    cfl_max<DIM, FLAT, true>(a, geo, m, rec, rec32, Pc, seen, rate_max);
   }
+  const double w = warp_max_d(rate_max);
+  if ((threadIdx.x & 31u) == 0) atomicMax(a.smax_out, (unsigned long long)__double_as_longlong(w));
 }
 
 __global__ void __launch_bounds__(256) ct_copy_kernel(int nblocks, CtGeom g, const double* __restrict__ src, double* dst,
                                                       int to_ring) {
-  const long long n = (long long)nblocks * g.nown_b;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / g.nown_b);
+  const unsigned n = (unsigned)nblocks * (unsigned)g.nown_b;  // below the ring-extended count, which fits 31 bits
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const int b = (int)(t / (unsigned)g.nown_b);
     int d, i, j, k;
-    owned_face(g, (int)(t - (long long)b * g.nown_b), d, i, j, k);
+    owned_face(g, (int)(t - (unsigned)b * (unsigned)g.nown_b), d, i, j, k);
     const long long o = (long long)b * g.nfb + ring_index(g, d, i, j, k);
     if (to_ring)
       dst[o] = src[t];
@@ -933,12 +968,15 @@ cudaError_t launch_ct_stage(const StageArgs& a, const CtArgs& c, bool mixed, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_ct_cell_field(const StageArgs& a, const CtArgs& c, double* P, float* P32, cudaStream_t st) {
-  const long long nc = (long long)a.nblocks * a.nint;
+cudaError_t launch_ct_load(const StageArgs& a, const CtArgs& c, double* P, float* P32, double* U, cudaStream_t st) {
+  int grid = grid_of((long long)a.nblocks * a.nint) / 4;  // about eight CTAs per SM: few atomics on the one rate word
+  if (grid < 1) grid = 1;
   if (a.ndim == 3)
-    ct_cell_field_kernel<3><<<grid_of(nc), 256, 0, st>>>(a, c, P, P32);
+    a.flat ? ct_load_kernel<3, true><<<grid, 256, 0, st>>>(a, c, P, P32, U)
+           : ct_load_kernel<3, false><<<grid, 256, 0, st>>>(a, c, P, P32, U);
   else
-    ct_cell_field_kernel<2><<<grid_of(nc), 256, 0, st>>>(a, c, P, P32);
+    a.flat ? ct_load_kernel<2, true><<<grid, 256, 0, st>>>(a, c, P, P32, U)
+           : ct_load_kernel<2, false><<<grid, 256, 0, st>>>(a, c, P, P32, U);
   return cudaGetLastError();
 }
 

@@ -104,9 +104,9 @@ cudaError_t launch_ct_ring_mean(const long long* dst, const long long* src, long
                                 cudaStream_t st);
 // mixed: FP32 face fluxes and cell sources (the mixed form); else FP64
 cudaError_t launch_ct_stage(const StageArgs& a, const CtArgs& c, bool mixed, cudaStream_t st);
-// B^d of the interior cells of P (and of its FP32 copy P32 when not null) from
-// the faces, psi = 0 (after a face load)
-cudaError_t launch_ct_cell_field(const StageArgs& a, const CtArgs& c, double* P, float* P32, cudaStream_t st);
+// after a face load: B^d of the interior cells of P (and of its FP32 copy P32
+// when not null) from the faces, psi = 0, then U and the CFL rate into a.smax_out
+cudaError_t launch_ct_load(const StageArgs& a, const CtArgs& c, double* P, float* P32, double* U, cudaStream_t st);
 // owned faces <-> the ring layout
 cudaError_t launch_ct_copy_faces(const StageArgs& a, const CtGeom& g, const double* src, double* dst, int to_ring,
                                  cudaStream_t st);

@@ -89,8 +89,7 @@ struct MetricArgs {
 };
 cudaError_t launch_metric_tables(const MetricArgs& m, cudaStream_t st);
 
-// interior <-> ghosted copies and the conserved state of loaded primitives
+// interior primitives out of the ghosted array
 cudaError_t launch_gather_interior(const StageArgs& a, const double* P, double* dst, cudaStream_t st);
-cudaError_t launch_init_cons(const StageArgs& a, const double* P, double* U, cudaStream_t st);
 
 }  // namespace bhac

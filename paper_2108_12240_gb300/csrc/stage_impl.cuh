@@ -498,7 +498,7 @@ __device__ __forceinline__ void cfl_max(const StageArgs& a, const LevelGeo& geo,
 }
 // the rate already in the result (0 where none is wanted)
 __device__ __forceinline__ unsigned long long cfl_seen(const StageArgs& a) {
-  return a.ch < 1.0 ? *reinterpret_cast<volatile unsigned long long*>(a.smax_out) : 0ull;
+  return a.ch < 1.0 && a.smax_out ? *reinterpret_cast<volatile unsigned long long*>(a.smax_out) : 0ull;
 }
 
 // ----------------------------------------------------------------------------
@@ -1641,8 +1641,8 @@ __global__ void __launch_bounds__(256) cfl_kernel(StageArgs a) {
 // Loading a state in one pass: the interior primitives src ([block][var][cell],
 // FP64) go to the ghosted FP64 array P and (mixed form) its FP32 copy P32; the
 // densitized conserved state U follows from them, and the CFL rate of the
-// loaded primitives is reduced into smax_out (the same per-cell rate as
-// cfl_kernel's).  Same loop as cfl_kernel.
+// loaded primitives is reduced into smax_out unless that is null (the same
+// per-cell rate as cfl_kernel's).  Same loop as cfl_kernel.
 template <int DIM, bool FLAT>
 __global__ void __launch_bounds__(256) load_kernel(StageArgs a, const double* __restrict__ src, double* P, float* P32,
                                                    double* U) {
@@ -1676,8 +1676,9 @@ __global__ void __launch_bounds__(256) load_kernel(StageArgs a, const double* __
     cons_direct(m, Pc, a.gam_fac, Uc);
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[((size_t)b * NV + v) * a.nint + ci] = FLAT ? Uc[v] : sg * Uc[v];
-    cfl_max<DIM, FLAT, true>(a, geo, m, rec, rec32, Pc, seen, rate_max);
+    if (a.smax_out) cfl_max<DIM, FLAT, true>(a, geo, m, rec, rec32, Pc, seen, rate_max);
   }
+  if (!a.smax_out) return;
   const double w = warp_max_d(rate_max);
   if ((threadIdx.x & 31u) == 0) atomicMax(a.smax_out, (unsigned long long)__double_as_longlong(w));
 }
