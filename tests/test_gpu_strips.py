@@ -28,3 +28,27 @@ def test_odd_blocks_2d_torus(gb, nx, form, tol):  # noqa: F811
     g = pb.torus_2d().with_(nx=(*nx, 1), nroot=(4, 4, 1), blocks=None)
     s, o, _ = one_step(gb, g, pb.fm_torus_prims(g), form)
     assert_parity(s.cons(), o.cons(), tol, f"{nx} {form}", g)
+
+
+@pytest.mark.parametrize("form,tol", [("fp64", TOL64), ("mixed", TOLMIX)])
+@pytest.mark.parametrize("nx,ndim", [((3, 4, 5), 3), ((7, 6, 3), 3), ((17, 5, 4), 3), ((70, 3, 1), 2), ((5, 130, 1), 2)])
+def test_constrained_transport_lines(gb, nx, ndim, form, tol):  # noqa: F811
+    """Lines of the face-flux kernel below and above one segment (64 faces),
+    CTAs whose lines span blocks, and remainders of the strips."""
+    import numpy as np
+
+    import oracle
+    from problems import ct
+    g = pb.periodic_box(ndim=ndim).with_(nx=nx, nroot=(2, 2, 2 if ndim == 3 else 1), blocks=None, divb="ct")
+    P, F = pb.random_periodic_prims(g), ct.random_potential_faces(g)
+    P[:, 8] = 0.0
+    s, o = gb.Solver(g, form), oracle.Oracle(g)
+    for x in (s, o):
+        x.set_prims(P)
+        x.set_faces(F)
+    dt = o.cfl_dt()
+    for x in (s, o):
+        x.step(dt)
+    assert_parity(s.cons(), o.cons(), tol, f"{nx} {form}", g)
+    ref = o.faces()
+    assert np.abs(s.faces() - ref).max() <= tol * np.abs(ref).max()
