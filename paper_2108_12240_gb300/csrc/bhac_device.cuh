@@ -590,6 +590,24 @@ BHAC_HD T ppm_iface(T am1, T a0, T a1, T a2) {
   return v;
 }
 
+// FP32: the same clipping by min and max that pass NaNs on, four instructions
+// where compares and selects take seven (mixed step of the 512x128x128 torus
+// 0.8% shorter; the bits are the same but for the sign of a zero).
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float ppm_iface(float am1, float a0, float a1, float a2) {
+  const float v = float(7.0 / 12.0) * (a0 + a1) - float(1.0 / 12.0) * (am1 + a2);
+  return min_nan(max_nan(v, fminf(a0, a1)), fmaxf(a0, a1));
+}
+
 template <typename T>
 BHAC_HD void ppm_limit(T a, T& aL, T& aR) {
   if (le0_t((aR - a) * (a - aL))) {
