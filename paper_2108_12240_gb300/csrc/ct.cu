@@ -477,6 +477,25 @@ __device__ __forceinline__ double emf2x4(const CtArgs& c, int b, int i, int j, i
 }
 
 
+// Four times the change of E_A from the edge at (i, j, k) to the next along e.
+// E_A = (F^q(B^p) - F^p(B^q)) / 4 summed over the four faces around the edge,
+// (p, q) the next directions after A: two flux arrays, whose elements are
+// addressed by strides from the edge's (16 separate indices took most of the
+// kernel's instructions).
+template <int A>
+__device__ __forceinline__ double emf_diff(const CtArgs& c, int b, int i, int j, int k, int e) {
+  constexpr int p = (A + 1) % 3, q = (A + 2) % 3;  // E_3: p = 1, q = 2 (1-based)
+  const CtGeom& g = c.g;
+  const int sp[3] = {1, g.fe[p][0], g.fe[p][0] * g.fe[p][1]};  // strides of the arrays of direction p, q
+  const int sq[3] = {1, g.fe[q][0], g.fe[q][0] * g.fe[q][1]};
+  const double* X = c.xf + (long long)b * NV * g.nfb;
+  const double* Q = X + NV * g.foff[q] + (B1 + p) * g.nfd[q] + (k + g.fo[q][2]) * sq[2] + (j + g.fo[q][1]) * sq[1] + (i + g.fo[q][0]);
+  const double* P = X + NV * g.foff[p] + (B1 + q) * g.nfd[p] + (k + g.fo[p][2]) * sp[2] + (j + g.fo[p][1]) * sp[1] + (i + g.fo[p][0]);
+  const int oq = sel3(e, sq[0], sq[1], sq[2]), op = sel3(e, sp[0], sp[1], sp[2]);
+  const double lo = Q[0] + Q[-sq[p]] - P[0] - P[-sp[q]];
+  return (Q[oq] + Q[oq - sq[p]] - P[op] - P[op - sp[q]]) - lo;
+}
+
 // d_t Phi = -curl E and the stage combination, one thread per owned face.
 template <int DIM>
 __global__ void __launch_bounds__(256) ct_face_kernel(StageArgs a, CtArgs c) {
@@ -495,14 +514,13 @@ __global__ void __launch_bounds__(256) ct_face_kernel(StageArgs a, CtArgs c) {
     const double qx = 0.25 * a.idx[0], qy = 0.25 * a.idx[1], qz = 0.25 * a.idx[2];
     double R;
     if (d == 0) {
-      R = -(emf3x4(c, b, i, j + 1, k) - emf3x4(c, b, i, j, k)) * qy;
-      if (DIM == 3) R += (emf2x4(c, b, i, j, k + 1) - emf2x4(c, b, i, j, k)) * qz;
+      R = -emf_diff<2>(c, b, i, j, k, 1) * qy;
+      if (DIM == 3) R += emf_diff<1>(c, b, i, j, k, 2) * qz;
     } else if (d == 1) {
-      R = (emf3x4(c, b, i + 1, j, k) - emf3x4(c, b, i, j, k)) * qx;
-      if (DIM == 3) R -= (emf1x4(c, b, i, j, k + 1) - emf1x4(c, b, i, j, k)) * qz;
+      R = emf_diff<2>(c, b, i, j, k, 0) * qx;
+      if (DIM == 3) R -= emf_diff<0>(c, b, i, j, k, 2) * qz;
     } else {
-      R = -(emf2x4(c, b, i + 1, j, k) - emf2x4(c, b, i, j, k)) * qx +
-          (emf1x4(c, b, i, j + 1, k) - emf1x4(c, b, i, j, k)) * qy;
+      R = -emf_diff<1>(c, b, i, j, k, 0) * qx + emf_diff<0>(c, b, i, j, k, 1) * qy;
     }
     if (a.stage == 1)
       c.phi_out[o] = c.phi_in[o] + dt * R;
