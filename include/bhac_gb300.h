@@ -363,12 +363,12 @@ bhac_status bhac_launches_per_step(const bhac_ctx* ctx, int* launches);
  * warp-specialised form: p warps compute the next plane's face fluxes
  * while the others update the current plane's cells (0: the phased form).
  * tx, ty, threads, min_ctas = 0 keep the current setting.  Results do not
- * depend on the launch shape.  The default after bhac_init_grid: 256 threads,
- * one CTA per item, and the largest of the tiles 32x16, 16x16, 16x8, 8x8
+ * depend on the launch shape.  The default after bhac_init_grid: a thread per
+ * cell of the tile (64 to 256), one CTA per item, and the largest of the tiles 32x16, 16x16, 16x8, 8x8
  * that divides the block and fits the shared-memory limit (else the block's
  * face); in the mixed form the largest of them up to 16x16 that leaves room
- * for two CTAs per SM, with min_ctas = 2; smaller tiles and CTAs on a grid of
- * fewer tiles than four fifths of the SMs. */
+ * for two CTAs per SM, with min_ctas = 2; smaller tiles on a grid of fewer
+ * tiles than four fifths of the SMs. */
 bhac_status bhac_set_launch(bhac_ctx* ctx, int tx, int ty, int threads, int persistent, int min_ctas,
                             int producer_warps);
 

@@ -153,7 +153,7 @@ def default_shape(grid, precision: str, sms: int):
     nx, ny, nz = grid.nx
     mixed = precision == "mixed"
     limit = TWO_CTA_SMEM if mixed else SMEM_LIMIT
-    shape, threads = [nx, ny], 256
+    shape = [nx, ny]
     for tx, ty in ((32, 16), (16, 16), (16, 8), (8, 8)):
         if mixed and tx * ty > 256:
             continue
@@ -170,7 +170,6 @@ def default_shape(grid, precision: str, sms: int):
         if f <= 1 or shape[0] * shape[1] // f < 16:
             break
         shape[k] //= f
-        cells = shape[0] * shape[1]
-        threads = min(256, max(64, -(-cells // 32) * 32))
         two = two or (mixed and smem_bytes(*shape, grid.ndim, precision) <= limit)
+    threads = min(256, max(64, -(-shape[0] * shape[1] // 32) * 32))
     return (shape[0], shape[1], threads, 0, 2 if two else 1, 0)
