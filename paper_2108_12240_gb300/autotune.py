@@ -37,7 +37,7 @@ def smem_bytes(tx: int, ty: int, ndim: int, precision: str, producers: int = 0) 
 
 
 def candidates(grid, precision: str, include_ws: bool = False):
-    """Launch shapes to time.  160 threads (one-CTA register bound) lets two
+    """Launch shapes to time.  64 threads fit small tiles, 160 threads (one-CTA register bound) lets two
     CTAs of a ~190-register build share an SM with fewer idle threads in the
     last round of a phase than 128 or 256.  The warp-specialised form measured
     slower on every grid tried and is timed only on request."""
@@ -49,10 +49,10 @@ def candidates(grid, precision: str, include_ws: bool = False):
     for tx, ty in tiles:
         if smem_bytes(tx, ty, grid.ndim, precision) > SMEM_LIMIT:
             continue
-        for threads in (256, 160, 128):
-            if threads > 2 * tx * ty:
+        for threads in (256, 160, 128, 64):
+            if threads > 2 * tx * ty or (threads == 64 and tx * ty > 128):
                 continue
-            for minb in ((1, 2) if grid.ndim == 3 and threads != 160 else (1,)):
+            for minb in ((1, 2) if (grid.ndim == 3 or precision == "mixed") and threads != 160 else (1,)):
                 out.append((tx, ty, threads, 0, minb, 0))
     # the warp-specialised form (3-D): producer warps feed consumer warps
     if grid.ndim == 3 and include_ws:
