@@ -598,7 +598,9 @@ __global__ void __launch_bounds__(256) ct_face_level_kernel(StageArgs a, CtArgs 
 // the arithmetic of the sources (float in the mixed form, from the FP32
 // primitives and metric records).  Two CTAs per SM as the register bound (a
 // few spilled values; the mixed form's stage 2.5% faster than at one CTA).
-template <typename T, int DIM, bool FLAT>
+// NKM: the inversion's solver (0 analytic Newton, 1 Newton-Krylov), compiled in:
+// both in one kernel cost spilled registers.
+template <typename T, int DIM, bool FLAT, int NKM>
 __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) {
   const double dt = block_dt(a);
   if (a.stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *a.dt_dev = dt;
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(256, 2) ct_cell_kernel(StageArgs a, CtArgs c) 
       U[B1 + d] = half_t(c.phi_out[lo] + c.phi_out[hi]);
     }
     U[PSI] = 0.0;
-    finish_cell<T, DIM, FLAT, (sizeof(T) == 4), 2, true>(a, geo, b, ci, cg, I1, I2, U, cnt, rate_max);
+    finish_cell<T, DIM, FLAT, (sizeof(T) == 4), NKM, true>(a, geo, b, ci, cg, I1, I2, U, cnt, rate_max);
   }
   reduce_outputs(a, cnt, rate_max);
 }
@@ -1030,6 +1032,23 @@ static cudaError_t launch_ct_flux(const StageArgs& a, const CtArgs& c, const CtL
   return cudaGetLastError();
 }
 
+template <typename T, int DIM, bool FLAT>
+static void launch_ct_cell(const StageArgs& a, const CtArgs& c, int grid, cudaStream_t st) {
+  if (a.c2p_nk)
+    ct_cell_kernel<T, DIM, FLAT, 1><<<grid, 256, 0, st>>>(a, c);
+  else
+    ct_cell_kernel<T, DIM, FLAT, 0><<<grid, 256, 0, st>>>(a, c);
+}
+
+template <typename T>
+static cudaError_t launch_ct_cells(const StageArgs& a, const CtArgs& c, int grid, cudaStream_t st) {
+  if (a.ndim == 3)
+    a.flat ? launch_ct_cell<T, 3, true>(a, c, grid, st) : launch_ct_cell<T, 3, false>(a, c, grid, st);
+  else
+    a.flat ? launch_ct_cell<T, 2, true>(a, c, grid, st) : launch_ct_cell<T, 2, false>(a, c, grid, st);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_ct_stage(const StageArgs& a, const CtArgs& c, bool mixed, cudaStream_t st) {
   const long long no = (long long)a.nblocks * c.g.nown_b,
                   nc = (long long)a.nblocks * a.nint;
@@ -1054,22 +1073,7 @@ cudaError_t launch_ct_stage(const StageArgs& a, const CtArgs& c, bool mixed, cud
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (mixed) {
-    if (a.ndim == 3)
-      a.flat ? ct_cell_kernel<float, 3, true><<<grid_of(nc), 256, 0, st>>>(a, c)
-             : ct_cell_kernel<float, 3, false><<<grid_of(nc), 256, 0, st>>>(a, c);
-    else
-      a.flat ? ct_cell_kernel<float, 2, true><<<grid_of(nc), 256, 0, st>>>(a, c)
-             : ct_cell_kernel<float, 2, false><<<grid_of(nc), 256, 0, st>>>(a, c);
-  } else {
-    if (a.ndim == 3)
-      a.flat ? ct_cell_kernel<double, 3, true><<<grid_of(nc), 256, 0, st>>>(a, c)
-             : ct_cell_kernel<double, 3, false><<<grid_of(nc), 256, 0, st>>>(a, c);
-    else
-      a.flat ? ct_cell_kernel<double, 2, true><<<grid_of(nc), 256, 0, st>>>(a, c)
-             : ct_cell_kernel<double, 2, false><<<grid_of(nc), 256, 0, st>>>(a, c);
-  }
-  return cudaGetLastError();
+  return mixed ? launch_ct_cells<float>(a, c, grid_of(nc), st) : launch_ct_cells<double>(a, c, grid_of(nc), st);
 }
 
 cudaError_t launch_ct_load(const StageArgs& a, const CtArgs& c, double* P, float* P32, double* U, cudaStream_t st) {

@@ -12,6 +12,8 @@
 // next, so no interior face flux is evaluated twice.
 #pragma once
 
+#include <type_traits>
+
 #include "amr.h"
 #include "bhac_device.cuh"
 #include "launch.h"
@@ -137,82 +139,99 @@ BHAC_HD T c2p_f1d(const C2PQ<T>& q, T gf, T v2max, T Z) {
 
 // Momentum and energy residuals of the two-dimensional system in (Z, v^2):
 //   F1 = (Z + B^2)^2 v^2 - (B.S)^2 (2 Z + B^2) / Z^2 - S^2,
-//   F2 = Z - p + B^2 (1 + v^2)/2 - (B.S)^2 / (2 Z^2) - E.
+//   F2 = Z - p + B^2 (1 + v^2)/2 - (B.S)^2 / (2 Z^2) - E,
+// as f1 = F1 / 2 and f2 = F2 with the constants of c2p_newton_step_t.
 template <typename T>
-BHAC_HD void c2p_residual_t(const C2PQ<T>& q, T gf, T Z, T v2, T& F1, T& F2) {
+BHAC_HD void c2p_residual_t(const C2PQ<T>& q, T gf, T hB, T hS2, T hBS2, T ec, T gD, T Z, T v2, T& f1, T& f2) {
   const T omv = T(1.0) - v2;
   const T sq = omv * rsqrt_t(omv);
-  const T pr = gf * (Z * omv - q.D * sq);
   const T iZ = rcp_t(Z);
-  const T iZ2 = iZ * iZ;
-  const T BS2 = q.BS * q.BS;
+  const T h = mul_rn(hBS2, iZ * iZ);
   const T ZB = Z + q.Bsq;
-  F1 = ZB * ZB * v2 - BS2 * (T(2.0) * Z + q.Bsq) * iZ2 - q.S2;
-  F2 = Z - pr + T(0.5) * q.Bsq * (T(1.0) + v2) - T(0.5) * BS2 * iZ2 - q.E;
+  f1 = fma_t(-h, Z + ZB, fma_t(half_t(ZB) * ZB, v2, -hS2));
+  f2 = fma_t(gD, sq, fma_t(-mul_rn(gf, Z), omv, fma_t(hB, v2, Z + ec) - h));
 }
 
 // One Jacobian-free Newton-Krylov step at (Z, v^2): the system scaled by rows
-// 1/(Z + B^2)^2 and 1/Z, unknowns (dZ/Z, dv^2); GMRES, whose Krylov space is
+// 2/(Z + B^2)^2 and 1/Z, unknowns (dZ/Z, dv^2); GMRES, whose Krylov space is
 // the plane after two vectors, on products of the Jacobian with unit vectors
 // taken as forward differences with step 2^-26 (backward where the forward
-// point would leave 0 <= v^2 < 1).  Writes the step (dZ, dv^2).
-template <typename T>
-BHAC_HD void c2p_nk_step_t(const C2PQ<T>& q, T gf, T Z, T v2, T& dZ, T& dv2) {
-  const T eps = T(1.4901161193847656e-08), ieps = T(67108864.0);  // 2^-26, 2^26
+// point would leave 0 <= v^2 < 1).  Writes the step (dZ, dv^2).  LOW: the
+// Krylov algebra in FP32, the residuals and their differences in FP64 (about 92
+// FP64 instructions against 150): as in c2p_newton_step_t from the second step
+// on, where 1e-7 of the step does not reach the result.
+template <typename T, bool LOW>
+BHAC_HD void c2p_nk_step_t(const C2PQ<T>& q, T gf, T hB, T hS2, T hBS2, T ec, T gD, T Z, T v2, T& dZ, T& dv2) {
+  using A = typename std::conditional<LOW, typename LowOf<T>::type, T>::type;
+  auto dn = [](T x) -> A {
+    if constexpr (LOW) return low_t(x);
+    else return x;
+  };
+  auto up = [](A x) -> T {
+    if constexpr (LOW) return high_t(x, T(0));
+    else return x;
+  };
+  auto inv = [](A x) -> A {
+    if constexpr (LOW) return rcp_low(x);
+    else return rcp_t(x);
+  };
+  const T eps = T(1.4901161193847656e-08);  // 2^-26
+  const A ieps = A(67108864.0f);            // 2^26
   const T ZB = Z + q.Bsq;
-  const T rs0 = rcp_t(ZB * ZB), rs1 = rcp_t(Z);
+  const T rs0 = rcp_t(half_t(ZB) * ZB), rs1 = rcp_t(Z);
   T F1, F2;
-  c2p_residual_t(q, gf, Z, v2, F1, F2);
-  const T G1 = rs0 * F1, G2 = rs1 * F2;
-  const T beta = sqrt_t(G1 * G1 + G2 * G2);
+  c2p_residual_t(q, gf, hB, hS2, hBS2, ec, gD, Z, v2, F1, F2);
+  const T G1 = mul_rn(rs0, F1), G2 = mul_rn(rs1, F2);
+  const A g1 = dn(G1), g2 = dn(G2);
+  const A beta = sqrt_t(g1 * g1 + g2 * g2);
   dZ = T(0.0);
   dv2 = T(0.0);
   if (!gt0_t(beta)) return;
-  const T ib = rcp_t(beta);
-  const T a1 = -G1 * ib, a2 = -G2 * ib;  // first basis vector
-  // J a by a one-sided difference
-  T sgn = T(1.0);
-  {
-    const T w = v2 + eps * a2;
-    if (lt0_x(w) || le_x(T(1.0), w)) sgn = T(-1.0);
-  }
-  T P1, P2;
-  c2p_residual_t(q, gf, Z + sgn * eps * a1 * Z, v2 + sgn * eps * a2, P1, P2);
-  T j1 = (rs0 * P1 - G1) * (sgn * ieps), j2 = (rs1 * P2 - G2) * (sgn * ieps);
-  const T h11 = j1 * a1 + j2 * a2;
+  // the scaled Jacobian times the unit vector (u1, u2) by a one-sided difference
+  auto product = [&](A u1, A u2, A& j1, A& j2) {
+    const T w1 = up(u1), w2 = up(u2);
+    const T w = fma_t(eps, w2, v2);
+    const bool back = lt0_x(w) || le_x(T(1.0), w);
+    const T e = back ? -eps : eps;
+    T P1, P2;
+    c2p_residual_t(q, gf, hB, hS2, hBS2, ec, gD, fma_t(mul_rn(Z, w1), e, Z), back ? fma_t(e, w2, v2) : w, P1, P2);
+    const A s = back ? -ieps : ieps;
+    j1 = dn(fma_t(rs0, P1, -G1)) * s;
+    j2 = dn(fma_t(rs1, P2, -G2)) * s;
+  };
+  const A ib = inv(beta);
+  const A a1 = -g1 * ib, a2 = -g2 * ib;  // first basis vector
+  A j1, j2;
+  product(a1, a2, j1, j2);
+  const A h11 = j1 * a1 + j2 * a2;
   j1 = j1 - h11 * a1;
   j2 = j2 - h11 * a2;
-  const T h21 = sqrt_t(j1 * j1 + j2 * j2);
-  if (!lt_t(T(1e-14) * abs_t(h11), h21)) {  // a spans an invariant direction
-    const T y = beta * rcp_t(h11);
-    dZ = mul_rn(Z, y * a1);
-    dv2 = mul_rn(y, a2);
+  const A h21 = sqrt_t(j1 * j1 + j2 * j2);
+  if (!lt_t(A(LOW ? 1e-6f : 1e-14f) * abs_t(h11), h21)) {  // a spans an invariant direction
+    const A y = beta * inv(h11);
+    dZ = mul_rn(Z, up(y * a1));
+    dv2 = up(mul_rn(y, a2));
     return;
   }
-  const T i21 = rcp_t(h21);
-  const T b1 = j1 * i21, b2 = j2 * i21;  // second basis vector
-  sgn = T(1.0);
-  {
-    const T w = v2 + eps * b2;
-    if (lt0_x(w) || le_x(T(1.0), w)) sgn = T(-1.0);
-  }
-  c2p_residual_t(q, gf, Z + sgn * eps * b1 * Z, v2 + sgn * eps * b2, P1, P2);
-  T k1 = (rs0 * P1 - G1) * (sgn * ieps), k2 = (rs1 * P2 - G2) * (sgn * ieps);
-  const T h12 = k1 * a1 + k2 * a2;
+  const A i21 = inv(h21);
+  const A b1 = j1 * i21, b2 = j2 * i21;  // second basis vector
+  A k1, k2;
+  product(b1, b2, k1, k2);
+  const A h12 = k1 * a1 + k2 * a2;
   k1 = k1 - h12 * a1;
   k2 = k2 - h12 * a2;
-  const T h22 = k1 * b1 + k2 * b2;
+  const A h22 = k1 * b1 + k2 * b2;
   // min |beta e1 - H y| for the 2 x 2 Hessenberg H: a Givens rotation, then
   // back substitution
-  const T r = sqrt_t(h11 * h11 + h21 * h21);
-  const T ir = rcp_t(r);
-  const T c = h11 * ir, sn = h21 * ir;
-  const T R12 = c * h12 + sn * h22;
-  const T R22 = -sn * h12 + c * h22;
-  const T y1 = (-sn * beta) * rcp_t(R22);
-  const T y0 = (c * beta - R12 * y1) * ir;
-  dZ = mul_rn(Z, y0 * a1 + y1 * b1);
-  dv2 = mul_rn(y0, a2) + mul_rn(y1, b2);
+  const A r = sqrt_t(h11 * h11 + h21 * h21);
+  const A ir = inv(r);
+  const A c = h11 * ir, sn = h21 * ir;
+  const A R12 = c * h12 + sn * h22;
+  const A R22 = -sn * h12 + c * h22;
+  const A y1 = (-sn * beta) * inv(R22);
+  const A y0 = (c * beta - R12 * y1) * ir;
+  dZ = mul_rn(Z, up(y0 * a1 + y1 * b1));
+  dv2 = up(mul_rn(y0, a2) + mul_rn(y1, b2));
 }
 
 // One Newton step at (Z, v^2) of f1 = F1 / 2 and f2 = F2, with the constants
@@ -315,7 +334,10 @@ BHAC_HD int con2prim_t(const Met<T>& m, const T* U, const T* Pg, size_t ps, T Z0
     for (int it = 0; it < maxit; ++it) {
       T dZ, dv2;
       if (NKM == 1 || (NKM == 2 && nk)) {
-        c2p_nk_step_t(q, gf, Z, v2, dZ, dv2);
+        if (it >= 1 && it <= 3)
+          c2p_nk_step_t<T, true>(q, gf, hB, hS2, hBS2, ec, gD, Z, v2, dZ, dv2);
+        else
+          c2p_nk_step_t<T, false>(q, gf, hB, hS2, hBS2, ec, gD, Z, v2, dZ, dv2);
       } else {
         c2p_newton_step_t(q, gf, hB, hS2, hBS2, ec, gD, hgD, Z, v2, it >= 1 && it <= 3, dZ, dv2);
       }
