@@ -122,6 +122,31 @@ struct HostState {
   std::vector<float> tc32, tf132, tf232;
 };
 
+// recon_edges with the operations of one cell of a long strip counted: its
+// difference to the next cell and the interface value there once, since both
+// are shared with that cell.
+template <typename T>
+void edges_once(int recon, T s_m2, T s_m1, T s0, T s1, T s2, T& aL, T& aR) {
+  const bool on = g_on;
+  if (recon != 0) {
+    recon_edges(recon, s_m2, s_m1, s0, s1, s2, aL, aR);
+  } else if constexpr (PpmByDifferences<T>::value) {
+    g_on = false;
+    const T d0 = s_m1 - s_m2, d1 = s0 - s_m1, d3 = s2 - s1, w = ppm_dev(d0, d1, s1 - s0);
+    g_on = on;
+    T r = ppm_dev(d1, s1 - s0, d3), l = w - d1;
+    limit_dev(l, r);
+    aL = s0 + l;
+    aR = s0 + r;
+  } else {
+    g_on = false;
+    aL = ppm_iface(s_m2, s_m1, s0, s1);
+    g_on = on;
+    aR = ppm_iface(s_m1, s0, s1, s2);
+    ppm_limit(s0, aL, aR);
+  }
+}
+
 template <typename T, typename S>
 void load_stencil(const StageArgs& a, const S* Pb, int d, int ig, int jg, int kg, T PL[NV], T PR[NV]) {
   const int sd = d == 0 ? 1 : (d == 1 ? a.Nx : a.Nx * a.Ny);
@@ -136,7 +161,7 @@ void load_stencil(const StageArgs& a, const S* Pb, int d, int ig, int jg, int kg
     g_on = false;
     recon_edges(a.recon, T(p[-3 * sd]), T(p[-2 * sd]), T(p[-sd]), T(p[0]), T(p[sd]), l0, r0);
     g_on = on;
-    recon_edges(a.recon, T(p[-2 * sd]), T(p[-sd]), T(p[0]), T(p[sd]), T(p[2 * sd]), l1, r1);
+    edges_once(a.recon, T(p[-2 * sd]), T(p[-sd]), T(p[0]), T(p[sd]), T(p[2 * sd]), l1, r1);
     PL[v] = r0;
     PR[v] = l1;
   }
