@@ -191,6 +191,7 @@ BHAC_HD Met<T> load_centre_metric(const R* __restrict__ rec) {
 template <typename T>
 BHAC_HD T fma_t(T a, T b, T c) { return a * b + c; }
 BHAC_HD double fma_t(double a, double b, double c) { return fma(a, b, c); }
+BHAC_HD float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 template <typename T>
 BHAC_HD T mul_rn(T a, T b) {
   return a * b;
@@ -199,6 +200,14 @@ template <>
 BHAC_HD double mul_rn<double>(double a, double b) {
 #ifdef __CUDA_ARCH__
   return __dmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+template <>
+BHAC_HD float mul_rn<float>(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
 #else
   return a * b;
 #endif
