@@ -358,9 +358,13 @@ __device__ __forceinline__ double sqrt_t(double x) {
 }
 __device__ __forceinline__ double high_t(float x, double) { return widen_f32(x); }
 __device__ __forceinline__ float rcp_low(float x) { return rcp_approx_f32(x); }
-// magnitude within 2^-50 .. 2^50: products of a few such values stay in FP32's range
+// magnitude within 2^-36 .. 2^50: what an FP32 solve of the inversion forms stays
+// in FP32's range.  The momentum residual is of the size of (Z + B^2)^2 / 2 times
+// its relative error; from 2^-36 on that expression's own rounding (2^-53 of it)
+// is not below the smallest normal FP32 value, 2^-126, so no part of a residual
+// above the rounding is flushed to zero.
 __device__ __forceinline__ bool low_range_t(double x) {
-  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) - 973u * kHiOne < 100u * kHiOne;
+  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) - 987u * kHiOne < 86u * kHiOne;
 }
 __device__ __forceinline__ double to_double(double x) { return x; }
 __device__ __forceinline__ double to_double(float x) { return widen_f32(x); }

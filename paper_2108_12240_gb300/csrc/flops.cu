@@ -81,7 +81,7 @@ inline N64 half_t(N64 x) {
 inline N32 low_t(N64 x) { return N32((float)x.v); }
 inline N64 high_t(N32 x, N64) { return N64((double)x.v); }
 inline N32 rcp_low(N32 x) { return rcp_t(x); }
-inline bool low_range_t(N64 x) { return std::fabs(x.v) > 0x1p-50 && std::fabs(x.v) < 0x1p50; }
+inline bool low_range_t(N64 x) { return std::fabs(x.v) >= 0x1p-36 && std::fabs(x.v) < 0x1p50; }
 inline void limit_dev(N64& l, N64& r) {  // integer decisions and results
   if (!(l.v * r.v < 0.0)) {
     l.v = r.v = 0.0;

@@ -87,6 +87,14 @@ def check(gb, rho, p_over_rho, sigma, u, c2p, form, spread=0.2):  # noqa: F811
     assert np.all(err <= bar[ok]), (float((err / bar[ok]).max()), float((err / p[ok]).max()))
 
 
+# (products of two 1e-30 densities leave the FP32 range of the mixed form's fluxes)
+@pytest.mark.parametrize("rho,form", [(r, f) for r in (1.0, 1e-11, 1e-13, 1e-14, 2e-15, 1e-16, 1e-30)
+                                      for f in ("fp64", "mixed") if not (r < 1e-20 and f == "mixed")])
+@pytest.mark.parametrize("c2p", ["newton", "nk"])
+def test_small_densities(gb, rho, c2p, form):  # noqa: F811
+    check(gb, rho, 1e-2, 0.1, 0.3, c2p, form)
+
+
 @pytest.mark.parametrize("form", ["fp64", "mixed"])
 @pytest.mark.parametrize("c2p", ["newton", "nk"])
 @pytest.mark.parametrize("sigma", [1e2, 1e3, 1e5])
