@@ -646,7 +646,10 @@ BHAC_HD T minmod_t(T a, T b) {
 // [0, d_i]; a cell's edges deviate from a by r = w at its high face and
 // l = w - d at its low face.  They have opposite signs unless the cell is a
 // local extremum (flat), and the CW84 overshoot conditions are |l| > 2 |r|
-// (then l = -2 r) and |r| > 2 |l| (then r = -2 l).  Halving, doubling, signs
+// (then l = -2 r) and |r| > 2 |l| (then r = -2 l).  A deviation that is still the
+// difference to the neighbour stands for a clipped interface value: that edge is
+// the neighbour's value itself (low_edge, high_edge), which a + (neighbour - a)
+// would round to a's own last place.  Halving, doubling, signs
 // and magnitudes of doubles are integer operations, so a cell costs 7 FP64
 // instructions in a strip of six (one per difference, three per interface,
 // two per cell) where the value form above costs 14 (19 without a strip); the
@@ -725,6 +728,36 @@ BHAC_HD T ppm_dev(T dm, T d, T dp) {
   return clip_dev(fma_t(dm - dp, T(1.0 / 12.0), half_t(d)), d);
 }
 
+// A cell's edges from its value a, its deviations l and r, and the neighbours nb
+// with their differences d to it (d = a - nb below, nb - a above).
+template <typename T>
+BHAC_HD T low_edge(T a, T l, T d, T nb) {
+  const T e = a + l;
+  return l < -d || -d < l ? e : nb;
+}
+template <typename T>
+BHAC_HD T high_edge(T a, T r, T d, T nb) {
+  const T e = a + r;
+  return r < d || d < r ? e : nb;
+}
+// (bit compares on the device: a difference passes clip_dev and 0 - d unchanged)
+BHAC_HD double low_edge(double a, double l, double d, double nb) {
+#ifdef __CUDA_ARCH__
+  const bool at = (__double2hiint(l) ^ __double2hiint(d)) == (int)0x80000000 && __double2loint(l) == __double2loint(d);
+  return at ? nb : a + l;
+#else
+  return low_edge<double>(a, l, d, nb);
+#endif
+}
+BHAC_HD double high_edge(double a, double r, double d, double nb) {
+#ifdef __CUDA_ARCH__
+  const bool at = __double2hiint(r) == __double2hiint(d) && __double2loint(r) == __double2loint(d);
+  return at ? nb : a + r;
+#else
+  return high_edge<double>(a, r, d, nb);
+#endif
+}
+
 // Both edges of one cell from its five-point stencil s_m2..s2 (cells c-2..c+2):
 // aL at the cell's low face, aR at its high face.  The same formulas as
 // recon_var evaluates per face, so a face's states from two cells' edges are
@@ -736,8 +769,8 @@ BHAC_HD void recon_edges(int recon, T s_m2, T s_m1, T s0, T s1, T s2, T& aL, T& 
       const T d0 = s_m1 - s_m2, d1 = s0 - s_m1, d2 = s1 - s0, d3 = s2 - s1;
       T l = ppm_dev(d0, d1, d2) - d1, r = ppm_dev(d1, d2, d3);
       limit_dev(l, r);
-      aL = s0 + l;
-      aR = s0 + r;
+      aL = low_edge(s0, l, d1, s_m1);
+      aR = high_edge(s0, r, d2, s1);
     } else {
       aL = ppm_iface(s_m2, s_m1, s0, s1);
       aR = ppm_iface(s_m1, s0, s1, s2);
@@ -759,8 +792,8 @@ BHAC_HD void recon_var(int recon, T a0, T a1, T a2, T a3, T a4, T a5, T& L, T& R
       T l2 = ppm_dev(d0, d1, d2) - d1, r2 = w, l3 = w - d2, r3 = ppm_dev(d2, d3, d4);
       limit_dev(l2, r2);
       limit_dev(l3, r3);
-      L = a2 + r2;
-      R = a3 + l3;
+      L = high_edge(a2, r2, d2, a3);
+      R = low_edge(a3, l3, d2, a2);
     } else {
       T l2 = ppm_iface(a0, a1, a2, a3);
       T r2 = ppm_iface(a1, a2, a3, a4);

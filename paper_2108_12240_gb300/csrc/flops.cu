@@ -134,10 +134,11 @@ void edges_once(int recon, T s_m2, T s_m1, T s0, T s1, T s2, T& aL, T& aR) {
     g_on = false;
     const T d0 = s_m1 - s_m2, d1 = s0 - s_m1, d3 = s2 - s1, w = ppm_dev(d0, d1, s1 - s0);
     g_on = on;
-    T r = ppm_dev(d1, s1 - s0, d3), l = w - d1;
+    const T d2 = s1 - s0;
+    T r = ppm_dev(d1, d2, d3), l = w - d1;
     limit_dev(l, r);
-    aL = s0 + l;
-    aR = s0 + r;
+    aL = low_edge(s0, l, d1, s_m1);
+    aR = high_edge(s0, r, d2, s1);
   } else {
     g_on = false;
     aL = ppm_iface(s_m2, s_m1, s0, s1);

@@ -947,8 +947,8 @@ __device__ __forceinline__ void strip_edges(int recon, const T* __restrict__ p, 
       T l = w - d[m + 1], r = wn;
       limit_dev(l, r);
       if (m < n) {
-        L[m * so] = q[m + 2] + l;
-        R[m * so] = q[m + 2] + r;
+        L[m * so] = low_edge(q[m + 2], l, d[m + 1], q[m + 1]);
+        R[m * so] = high_edge(q[m + 2], r, d[m + 2], q[m + 3]);
       }
       w = wn;
     }
