@@ -362,7 +362,8 @@ bhac_status bhac_launches_per_step(const bhac_ctx* ctx, int* launches);
  * kernel), and producer_warps = p > 0 (3-D only, p * 32 < threads) for the
  * warp-specialised form: p warps compute the next plane's face fluxes
  * while the others update the current plane's cells (0: the phased form).
- * tx, ty, threads, min_ctas = 0 keep the current setting.  Results do not
+ * tx, ty, threads, min_ctas = 0 keep the current setting (threads = 0 with a tile
+ * or producer warps means 256 until a size has been set).  Results do not
  * depend on the launch shape.  The default after bhac_init_grid: a thread per
  * cell of the tile (64 to 256), one CTA per item, and the largest of the tiles 32x16, 16x16, 16x8, 8x8
  * that divides the block and fits the shared-memory limit (else the block's

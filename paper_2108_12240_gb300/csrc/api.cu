@@ -426,6 +426,7 @@ void default_shape(bhac_ctx* c) {
   // 16x8 tiles of 32x24x16 blocks: 5.16, 4.78 and 5.13 ms)
   const int cells = c->tx * c->ty;
   c->threads = cells >= 256 ? 256 : (cells < 64 ? 64 : (cells + 31) / 32 * 32);
+  c->threads_auto = true;
 }
 
 // Z parts per (block, tile) column of the phased 3-D stage kernel.  A fixed
@@ -1107,9 +1108,13 @@ bhac_status bhac_get_c2p_status(bhac_ctx* c, unsigned char* out, int on_device) 
 bhac_status bhac_set_launch(bhac_ctx* c, int tx, int ty, int threads, int persistent, int min_ctas,
                             int producer_warps) {
   if (!c || min_ctas < 0 || min_ctas > 3 || producer_warps < 0) return BHAC_ERR_ARG;
-  if (producer_warps > 0 && (c->d.ndim != 3 || producer_warps * 32 >= (threads > 0 ? threads : c->threads)))
-    return BHAC_ERR_ARG;
-  const int ntx = tx > 0 ? tx : c->tx, nty = ty > 0 ? ty : c->ty, nth = threads > 0 ? threads : c->threads;
+  // threads not given: what is set stays; while that is still the default, a call
+  // that sets a tile or producer warps gets 256, since the default's CTA size was
+  // chosen for the default's tile in the phased form
+  const bool asks = tx > 0 || ty > 0 || producer_warps > 0;
+  const int nth = threads > 0 ? threads : (asks && c->threads_auto ? 256 : c->threads);
+  const int ntx = tx > 0 ? tx : c->tx, nty = ty > 0 ? ty : c->ty;
+  if (producer_warps > 0 && (c->d.ndim != 3 || producer_warps * 32 >= nth)) return BHAC_ERR_ARG;
   if (c->d.nx[0] % ntx || c->d.nx[1] % nty || nth % 32 || nth > 256 || persistent < 0 || persistent > 8)
     return BHAC_ERR_ARG;
   const size_t smem = stage_smem(c, ntx, nty, producer_warps);
@@ -1118,6 +1123,7 @@ bhac_status bhac_set_launch(bhac_ctx* c, int tx, int ty, int threads, int persis
   c->pwarps = producer_warps;
   c->tx = ntx;
   c->ty = nty;
+  if (threads > 0 || asks) c->threads_auto = false;
   c->threads = nth;
   c->persistent = persistent;
   c->nzp_eff = 0;

@@ -46,6 +46,7 @@ struct bhac_ctx {
   bool cfl_fresh;  // smax holds the CFL rate of the current primitives (set by loads and bhac_cfl_dt)
   // launch shape
   int tx, ty, threads, persistent, minb, pwarps;
+  bool threads_auto;  // the CTA size is still the default's
   // refinement levels: metric-table record offsets per level
   long long toff_c[bhac::MAXLEV], toff_f1[bhac::MAXLEV], toff_f2[bhac::MAXLEV];
   // cross-level ghost nodes (evaluated depth by depth) and flux correction
