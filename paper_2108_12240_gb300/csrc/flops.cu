@@ -201,7 +201,7 @@ void face(const StageArgs& a, const S* Pb, const R* tc, const R* tf1, const R* t
 // One cell through both stages' arithmetic; faces are counted once per
 // direction (the low face), as the kernel evaluates each face once.
 template <typename T, typename S, typename R>
-void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, double dt, int stage) {
+void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, double dt, int stage, bool screened) {
   const int bidx = h.ids[sb];
   const S* Pb;
   const R *tc, *tf1, *tf2;
@@ -324,9 +324,10 @@ void cell(const StageArgs& a, const HostState& h, int sb, int i, int j, int k, d
       for (int v = 0; v < NV; ++v) U[v] = N64(sg) * Uu[v];
     }
   }
-  // with ch >= 1 the rate is tabulated; below, the light-cone test leaves it
-  // out for nearly every cell of a curved grid
-  if (stage == 2 && a.flat && a.ch < 1.0) {
+  // with ch >= 1 the rate is tabulated; below, the stage kernel forms every
+  // cell's (the light-cone test that leaves it out on curved grids is in the
+  // constrained-transport, load and stand-alone reduction kernels only)
+  if (stage == 2 && a.ch < 1.0 && (a.flat || !screened)) {
     N64 acg[3] = {N64(1.0), N64(1.0), N64(1.0)};
     if (!a.flat) {
       acg[0] = N64(crec[C_ACG1]);
@@ -398,9 +399,9 @@ extern "C" bhac_status bhac_count_flops(bhac_ctx* c, double dt, int nsamples, un
     const int i = (int)(rng() % (unsigned)a.nx), j = (int)(rng() % (unsigned)a.ny), k = (int)(rng() % (unsigned)a.nz);
     for (int stage = 1; stage <= 2; ++stage) {
       if (c->mixed)
-        cell<N32, float, float>(a, h, sb, i, j, k, dt, stage);
+        cell<N32, float, float>(a, h, sb, i, j, k, dt, stage, c->ct);
       else
-        cell<N64, double, double>(a, h, sb, i, j, k, dt, stage);
+        cell<N64, double, double>(a, h, sb, i, j, k, dt, stage, c->ct);
     }
   }
   g_on = true;
