@@ -4,8 +4,9 @@ Candidates are CTA tiles (tx, ty) that divide the block, threads per CTA,
 the register bound of the 3-D kernel (one or two resident CTAs per SM) and
 the persistent work-queue schedule.  Each candidate is timed on the caller's
 own grid and state with CUDA events over a few device-dt steps; the fastest
-is applied and cached in a JSON file keyed by GPU name, block shape, level
-count, dimensionality and precision, so later runs skip the search.  Every
+is applied and cached in a JSON file keyed by GPU name, block shape and count
+(few blocks want smaller tiles), level count, dimensionality, precision and
+what selects another kernel, so later runs skip the search.  Every
 candidate gives bit-identical results (the launch shape changes only the
 order in which blocks are visited), so tuning never changes the answer.
 """
@@ -37,10 +38,10 @@ def smem_bytes(tx: int, ty: int, ndim: int, precision: str, producers: int = 0) 
 
 
 def candidates(grid, precision: str, include_ws: bool = False):
-    """Launch shapes to time.  64 threads fit small tiles, 160 threads (one-CTA register bound) lets two
-    CTAs of a ~190-register build share an SM with fewer idle threads in the
-    last round of a phase than 128 or 256.  The warp-specialised form measured
-    slower on every grid tried and is timed only on request."""
+    """Launch shapes to time (64 threads fit small tiles).  160 threads, once a way
+    to two CTAs of a ~190-register build, are 224 with the helper warps and were
+    13% or more behind the best shape on every grid tried; the warp-specialised
+    form measured slower too and is timed only on request."""
     nx, ny = grid.nx[0], grid.nx[1]
     tiles = [(tx, ty) for tx in (32, 16, 8) for ty in (16, 8, 4) if nx % tx == 0 and ny % ty == 0 and tx * ty >= 64]
     if not tiles:
@@ -49,10 +50,10 @@ def candidates(grid, precision: str, include_ws: bool = False):
     for tx, ty in tiles:
         if smem_bytes(tx, ty, grid.ndim, precision) > SMEM_LIMIT:
             continue
-        for threads in (256, 160, 128, 64):
+        for threads in (256, 128, 64):
             if threads > 2 * tx * ty or (threads == 64 and tx * ty > 128):
                 continue
-            for minb in ((1, 2) if (grid.ndim == 3 or precision == "mixed") and threads != 160 else (1,)):
+            for minb in ((1, 2) if grid.ndim == 3 or precision == "mixed" else (1,)):
                 out.append((tx, ty, threads, 0, minb, 0))
     # the warp-specialised form (3-D): producer warps feed consumer warps
     if grid.ndim == 3 and include_ws:
@@ -68,8 +69,8 @@ def candidates(grid, precision: str, include_ws: bool = False):
 def key_of(grid, precision: str) -> str:
     import torch
     name = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
-    return (f"{name}|{KERNEL_TAG}|nx={grid.nx[0]}x{grid.nx[1]}x{grid.nx[2]}|ndim={grid.ndim}"
-            f"|levels={grid.nlevels}|{precision}|{grid.recon}")
+    return (f"{name}|{KERNEL_TAG}|nx={grid.nx[0]}x{grid.nx[1]}x{grid.nx[2]}|blocks={grid.nb}|ndim={grid.ndim}"
+            f"|levels={grid.nlevels}|{precision}|{grid.recon}|{grid.c2p}")
 
 
 def load_cache(path: str = DEFAULT_CACHE) -> dict:
