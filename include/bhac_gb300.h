@@ -437,8 +437,10 @@ bhac_status bhac_count_flops(bhac_ctx* ctx, double dt, int nsamples, unsigned se
  * bit patterns; doubles in and around the float range; round-to-nearest ties;
  * neighbours one ulp apart; zeros, subnormals, infinities, NaNs) and writes the
  * number of disagreements per operation to out[11]: [0] a < b, [1] x > 0,
- * [2] x <= 0, [3] |a| < |b|, [4] a <= b and x < 0 (all IEEE, NaN operands
- * included), [5] isfinite, [6] double -> float (bitwise; NaN as NaN),
+ * [2] x <= 0, [3] |a| < |b| and the PPM limiter's clipping and overshoot rules
+ * on a pair, [4] a <= b and x < 0 (all IEEE, NaN operands included), [5] isfinite,
+ * |x| and the exact x / 2, [6] double -> float, rounded (bitwise; NaN as NaN) and
+ * truncated,
  * [7] float -> double; and the operands whose result lies farther than the
  * bound from the reference: [8] 1/x more than 1 ulp from the IEEE reciprocal,
  * [9] x^(-1/2) more than 2 ulp from CUDA's rsqrt, [10] sqrt x more than 2 ulp

@@ -685,8 +685,9 @@ BHAC_HD double clip_dev(double w, double d) {
 #ifdef __CUDA_ARCH__
   const unsigned wh = (unsigned)__double2hiint(w), wl = (unsigned)__double2loint(w);
   const unsigned dh = (unsigned)__double2hiint(d), dl = (unsigned)__double2loint(d);
-  const bool fin = (wh & kHiExp) != kHiExp, opp = (int)(wh ^ dh) < 0, big = mag_lt(dh, dl, wh, wl);
-  const unsigned rh = fin ? (opp ? 0u : (big ? dh : wh)) : wh, rl = fin ? (opp ? 0u : (big ? dl : wl)) : wl;
+  const bool num = (wh & 0x7FFFFFFFu) <= kHiExp;  // not NaN (arithmetic's are quiet)
+  const bool opp = (int)(wh ^ dh) < 0, big = mag_lt(dh, dl, wh, wl);
+  const unsigned rh = num ? (opp ? 0u : (big ? dh : wh)) : wh, rl = num ? (opp ? 0u : (big ? dl : wl)) : wl;
   return __hiloint2double((int)rh, (int)rl);
 #else
   return clip_dev<double>(w, d);

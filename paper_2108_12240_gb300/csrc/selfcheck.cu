@@ -66,6 +66,35 @@ __device__ long long ulp_dist(double x, double y) {
   return a > b ? a - b : b - a;
 }
 
+// PPM's clipping and limiting of deviations on the integer pipes against the
+// plain compares, where those neither underflow (l r) nor overflow (2 l, 2 r), no
+// deviation is subnormal (its doubling is off by up to 2^-1021) and no difference
+// d is NaN (its clipped w then is, too); the sign of a zero is free.
+__device__ bool same_value(double x, double y) { return x == y || (isnan(x) && isnan(y)); }
+__device__ bool bad_deviations(double a, double b) {
+  if (!isnan(b) && !same_value(clip_dev(a, b), clip_dev<double>(a, b))) return true;
+  if (!(fabs(a) < 0x1p1000 && fabs(b) < 0x1p1000)) return false;
+  if (a != 0.0 && b != 0.0 && !(fabs(a * b) >= 0x1p-1022 && fabs(a) >= 0x1p-1022 && fabs(b) >= 0x1p-1022)) return false;
+  double l0 = a, r0 = b, l1 = a, r1 = b;
+  limit_dev(l0, r0);
+  limit_dev<double>(l1, r1);
+  return !same_value(l0, l1) || !same_value(r0, r1);
+}
+
+// the truncated FP32 copy: round towards zero, values below the normal range 0,
+// from 2^128 on infinite (as NaN, whose callers test their results)
+__device__ unsigned low_bits(double x) {
+  const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
+  if (!(fabs(x) < 0x1p128)) return sign | 0x7F800000u;
+  return fabs(x) < 0x1p-126 ? sign : __float_as_uint(__double2float_rz(x));
+}
+
+// x / 2 wherever that is normal; zeros and non-finite values stay
+__device__ bool bad_half(double x) {
+  if (x == 0.0 || !isfinite(x)) return __double_as_longlong(half_t(x)) != __double_as_longlong(x);
+  return fabs(x) >= 0x1p-1021 && half_t(x) != 0.5 * x;
+}
+
 __global__ void check_kernel(long long n, unsigned long long seed, unsigned long long* bad) {
   unsigned long long loc[kChecks] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -78,11 +107,13 @@ __global__ void check_kernel(long long n, unsigned long long seed, unsigned long
     if (lt_t(a, b) != (a < b)) ++loc[0];
     if (gt0_t(a) != (a > 0.0)) ++loc[1];
     if (le0_t(a) != (a <= 0.0)) ++loc[2];
-    if (lt_abs_t(a, b) != (fabs(a) < fabs(b))) ++loc[3];
+    if (lt_abs_t(a, b) != (fabs(a) < fabs(b)) || bad_deviations(a, b)) ++loc[3];
     if (le_x(a, b) != (a <= b) || lt0_x(a) != (a < 0.0)) ++loc[4];
-    if (finite_t(a) != (bool)isfinite(a)) ++loc[5];
+    if (finite_t(a) != (bool)isfinite(a) || bad_half(a) || !same_value(abs_t(a), fabs(a))) ++loc[5];
     const float f1 = narrow_f64(a), f0 = __double2float_rn(a);
-    if (!(isnan(f1) && isnan(f0)) && __float_as_uint(f1) != __float_as_uint(f0)) ++loc[6];
+    if ((!(isnan(f1) && isnan(f0)) && __float_as_uint(f1) != __float_as_uint(f0)) ||
+        __float_as_uint(low_t(a)) != low_bits(a))
+      ++loc[6];
     const float g = __uint_as_float((unsigned)(hb >> 32));
     const double w1 = widen_f32(g), w0 = (double)g;
     if (!(isnan(w1) && isnan(w0)) && __double_as_longlong(w1) != __double_as_longlong(w0)) ++loc[7];
