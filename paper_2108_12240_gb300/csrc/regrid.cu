@@ -682,6 +682,7 @@ extern "C" bhac_status bhac_regrid_transfer(const bhac_ctx* old, bhac_ctx* fresh
   fresh->ucur = 0;
   fresh->prims_ok = true;
   fresh->cfl_ok = false;
+  fresh->cfl_fresh = false;  // a load before this left another state's rate
   if (ct) {
     fresh->pcur = 0;
     fresh->faces_ok = true;
