@@ -367,7 +367,7 @@ bhac_status bhac_launches_per_step(const bhac_ctx* ctx, int* launches);
  * depend on the launch shape.  The default after bhac_init_grid: a thread per
  * cell of the tile (64 to 256), one CTA per item, and the largest of the tiles 32x16, 16x16, 16x8, 8x8
  * that divides the block and fits the shared-memory limit (else the block's
- * face); in the mixed form the largest of them up to 16x16 that leaves room
+ * face, or the largest part of it that fits); in the mixed form the largest of them up to 16x16 that leaves room
  * for two CTAs per SM, with min_ctas = 2; smaller tiles on a grid of fewer
  * tiles than four fifths of the SMs. */
 bhac_status bhac_set_launch(bhac_ctx* ctx, int tx, int ty, int threads, int persistent, int min_ctas,

@@ -165,10 +165,12 @@ def default_shape(grid, precision: str, sms: int):
     parts = 1
     while grid.ndim == 3 and nz % (2 * parts) == 0 and nz // (2 * parts) >= 4:
         parts *= 2
-    while 5 * grid.nb * (nx // shape[0]) * (ny // shape[1]) * parts < 4 * sms:
+    while True:
+        fits = smem_bytes(*shape, grid.ndim, precision) <= SMEM_LIMIT
+        few = 5 * grid.nb * (nx // shape[0]) * (ny // shape[1]) * parts < 4 * sms
         k = 0 if shape[0] > shape[1] else 1
         f = next((f for f in range(2, shape[k]) if shape[k] % f == 0), shape[k])
-        if f <= 1 or shape[0] * shape[1] // f < 16:
+        if f <= 1 or (fits and (not few or shape[0] * shape[1] // f < 16)):
             break
         shape[k] //= f
         two = two or (mixed and smem_bytes(*shape, grid.ndim, precision) <= limit)

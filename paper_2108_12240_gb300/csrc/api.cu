@@ -378,7 +378,7 @@ int launch_threads(const bhac_ctx* c) {
 
 // The launch shape after bhac_init_grid.  The largest of these tiles that
 // divides the block and fits the shared-memory limit, else the whole block
-// face; the mixed form takes tiles of at most 256 cells whose workspace lets
+// face (divided the same way as below where that does not fit); the mixed form takes tiles of at most 256 cells whose workspace lets
 // two CTAs share an SM, with the two-CTA register bound.  That is the fastest
 // family on every grid large enough to fill the GPU.  A grid whose tiles (times
 // the z parts choose_nzp may cut) are fewer than 4/5 of the SMs gets smaller
@@ -413,10 +413,12 @@ void default_shape(bhac_ctx* c) {
       if (n % f == 0) return f;
     return n;
   };
-  while (5LL * c->nb * (nx[0] / c->tx) * (nx[1] / c->ty) * parts < 4LL * nsm) {
+  for (;;) {
+    const bool fits = stage_smem(c, c->tx, c->ty, 0) <= (size_t)kMaxDynSmem;
+    const bool few = 5LL * c->nb * (nx[0] / c->tx) * (nx[1] / c->ty) * parts < 4LL * nsm;
     int& side = c->tx > c->ty ? c->tx : c->ty;
     const int f = least_factor(side);
-    if (f <= 1 || c->tx * c->ty / f < 16) break;
+    if (f <= 1 || (fits && (!few || c->tx * c->ty / f < 16))) break;
     side /= f;
     if (c->mixed && stage_smem(c, c->tx, c->ty, 0) <= limit) c->minb = 2;
   }

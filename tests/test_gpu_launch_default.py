@@ -34,3 +34,18 @@ def test_refused(gb, shape):  # noqa: F811
     with pytest.raises(gb.BhacError) as e:
         s.set_launch(*shape)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("nx,nroot", [((24, 20, 4), (6, 6, 4)), ((50, 44, 1), (12, 12, 1)), ((23, 29, 3), (5, 6, 5))])
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_default_fits_any_block(gb, nx, nroot, form):  # noqa: F811
+    """Block faces that no standard tile divides and that are too large for the
+    shared memory as a whole, on grids of many blocks."""
+    from paper_2108_12240_gb300 import autotune
+    from tests.test_gpu_parity import TOL64, TOLMIX, assert_parity, one_step
+    g = pb.periodic_box(ndim=3 if nx[2] > 1 else 2).with_(nx=nx, nroot=nroot, blocks=None)
+    tx, ty = autotune.default_shape(g, form, 152)[:2]
+    assert nx[0] % tx == 0 and nx[1] % ty == 0
+    assert autotune.smem_bytes(tx, ty, g.ndim, form) <= autotune.SMEM_LIMIT
+    s, o, _ = one_step(gb, g, pb.random_periodic_prims(g), form)
+    assert_parity(s.cons(), o.cons(), TOL64 if form == "fp64" else TOLMIX, f"{nx} {form}", g)
